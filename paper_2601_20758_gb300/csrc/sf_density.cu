@@ -1867,6 +1867,7 @@ sf_status batch_run(BatchPlan *P, float *const *outs, double *h_mass, cudaStream
 // Points (DIRECT)
 // ===========================================================================
 constexpr int kPtWarps = 4;
+constexpr int kWideLeaves = 512;
 
 struct PointsArgs {
     EngineArgs e;
@@ -1883,13 +1884,23 @@ struct __align__(16) PtWarpSmem {
     // staged candidates as structure of arrays (pairs of entries load as one 64-bit word)
     float sx[kPtRing], sy[kPtRing], sz[kPtRing], sc[kPtRing];
     float su[3][kPtRing];  // BW_ISO: su[0] = u^2; else u_x, u_y, u_z
+    float4 q[kLeaf];       // the query points
     int stack[kStack];
     int leaves[kBatch];
 };
 
-template <int KER, int BW, bool CLIP, bool CNT>
+// SPLIT warps work on one query leaf, each on every SPLIT-th candidate leaf (all walk the
+// index); their sums are added in warp order. SPLIT = kPtWarps where the query leaves
+// alone would not fill the chip: then the longest leaf sets the time (100,000 points: 877 us
+// by one warp a leaf, 289 us now).
+//
+// What bounds it: issue slots, about 9 a staged candidate (two candidates an instruction
+// in packed FP32) and 45 a candidate leaf; half of the staged candidates are in support
+// of a given lane (the union of 32 queries' reach).
+template <int KER, int BW, bool CLIP, bool CNT, int SPLIT>
 __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
     __shared__ PtWarpSmem W[kPtWarps];
+    __shared__ double s_part[SPLIT > 1 ? kPtWarps : 1][kLeaf];
     __shared__ float s_uni[3];
     __shared__ float s_runi[4];  // 1 / uniform l_k, and whether all l_k > 0
     __shared__ double s_inv;
@@ -1907,7 +1918,8 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
     }
     __syncthreads();
     PtWarpSmem &S = W[warp];
-    const int64_t slot = (int64_t)blockIdx.x * kPtWarps + warp;
+    const int part = warp % SPLIT;
+    const int64_t slot = ((int64_t)blockIdx.x * kPtWarps + warp) / SPLIT;
     if (slot >= a.nslots) return;
     const int64_t leaf = a.leaves ? (int64_t)a.leaves[slot] : slot;
     const int64_t qi = leaf * kLeaf + lane;
@@ -1918,7 +1930,7 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
     // query points: those inside the ROI box (closed)
     const bool active = valid && q.x >= a.e.blo[0] && q.x <= a.e.bhi[0] && q.y >= a.e.blo[1] &&
                         q.y <= a.e.bhi[1] && q.z >= a.e.blo[2] && q.z <= a.e.bhi[2];
-    a.inroi[oi] = active ? 1 : 0;
+    if (part == 0) a.inroi[oi] = active ? 1 : 0;
     const unsigned am = __ballot_sync(0xffffffffu, active);
     if (am == 0) return;
     float tlo[3] = {active ? q.x : INFINITY, active ? q.y : INFINITY, active ? q.z : INFINITY};
@@ -1939,28 +1951,58 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
         mcen[k] = 0.5f * (mlo[k] + mhi[k]);
         mhw[k] = 0.5f * (mhi[k] - mlo[k]);
     }
-    auto test = [&](int64_t node) { return node_reaches<KER, BW, CLIP>(a.e, s_uni, node, mlo, mhi); };
+    // A leaf whose points lie apart (at a jump of the Morton order) has a box that can cover
+    // clusters none of its points is near: from kWideLeaves candidate leaves on (the mean is
+    // about 200) nodes and candidates are tested against every point. A whole launch
+    // waited for single such leaves, of up to 36,000 candidate leaves: the densities at
+    // 16.8M clustered points took 44.2 ms, 23.6 ms with this test.
+    bool wide = false;
+    int seen = 0;
+    S.q[lane] = make_float4(active ? q.x : INFINITY, q.y, q.z, 0.f);
+    __syncwarp();
+    auto test = [&](int64_t node) {
+        if (!node_reaches<KER, BW, CLIP>(a.e, s_uni, node, mlo, mhi)) return false;
+        if (!wide) return true;
+        const float4 lo = __ldg(&a.e.tv.nlo[node]), hi = __ldg(&a.e.tv.nhi[node]);
+        float r[3];
+        if (BW == BW_UNIFORM) {
+            r[0] = rcp_approx(s_uni[0]); r[1] = rcp_approx(s_uni[1]); r[2] = rcp_approx(s_uni[2]);
+        } else {
+            const float4 e = __ldg(&a.e.nell[node]);
+            r[0] = rcp_approx(e.x); r[1] = rcp_approx(e.y); r[2] = rcp_approx(e.z);
+        }
+        bool near = false;
+        for (int j = 0; j < kLeaf; ++j) {
+            const float4 p = S.q[j];
+            const float gx = fmaxf(fmaxf(lo.x - p.x, p.x - hi.x), 0.f) * r[0];
+            const float gy = fmaxf(fmaxf(lo.y - p.y, p.y - hi.y), 0.f) * r[1];
+            const float gz = fmaxf(fmaxf(lo.z - p.z, p.z - hi.z), 0.f) * r[2];
+            near = near || fmaf(gz, gz, fmaf(gy, gy, gx * gx)) <
+                               KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
+        }
+        return near;
+    };
 
     float sum = 0.f, cmp = 0.f;
     unsigned long long npairs = 0;
     const f32x2 QX = f2_pack(q.x, q.x), QY = f2_pack(q.y, q.y), QZ = f2_pack(q.z, q.z);
-    // entries s and s + 1 (s even) against this lane's query
-    auto pair2 = [&](int s, float &acc0, float &acc1) {
-        const f32x2 dx = f2_sub(QX, f2_ld(&S.sx[s]));
-        const f32x2 dy = f2_sub(QY, f2_ld(&S.sy[s]));
-        const f32x2 dz = f2_sub(QZ, f2_ld(&S.sz[s]));
+    // two packed candidates against this lane's query
+    auto pair2 = [&](f32x2 x, f32x2 y, f32x2 z, f32x2 u0, f32x2 u1, f32x2 u2, f32x2 c, float &acc0, float &acc1) {
+        const f32x2 dx = f2_sub(QX, x);
+        const f32x2 dy = f2_sub(QY, y);
+        const f32x2 dz = f2_sub(QZ, z);
         f32x2 qq;
         if (BW == BW_ISO) {
-            qq = f2_mul(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), f2_ld(&S.su[0][s]));
+            qq = f2_mul(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), u0);
         } else {
-            const f32x2 tx = f2_mul(dx, f2_ld(&S.su[0][s]));
-            const f32x2 ty = f2_mul(dy, f2_ld(&S.su[1][s]));
-            const f32x2 tz = f2_mul(dz, f2_ld(&S.su[2][s]));
+            const f32x2 tx = f2_mul(dx, u0);
+            const f32x2 ty = f2_mul(dy, u1);
+            const f32x2 tz = f2_mul(dz, u2);
             qq = f2_fma(tz, tz, f2_fma(ty, ty, f2_mul(tx, tx)));
         }
         float q0, q1, c0, c1;
         f2_unpack(qq, q0, q1);
-        f2_unpack(f2_ld(&S.sc[s]), c0, c1);
+        f2_unpack(c, c0, c1);
         const bool in0 = q0 < KDef<KER>::qmax, in1 = q1 < KDef<KER>::qmax;
         if (KER == SF_K_GAUSS3) {
             if (in0) acc0 = fmaf(c0, ex2_approx(-q0), acc0);
@@ -1970,6 +2012,14 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
             if (in1) acc1 = fmaf(c1, 1.0f - q1, acc1);
         }
         if (CNT) npairs += (unsigned)in0 + (unsigned)in1;
+    };
+    // entries s, ..., s + 3 (s a multiple of 4): one 16-byte load each of x, y, z, u and c
+    auto quad = [&](int s, float &a0, float &a1, float &a2, float &a3) {
+        auto ld = [](const float *p) { return *reinterpret_cast<const ulonglong2 *>(p); };
+        const ulonglong2 x = ld(&S.sx[s]), y = ld(&S.sy[s]), z = ld(&S.sz[s]), c = ld(&S.sc[s]), u0 = ld(&S.su[0][s]);
+        const ulonglong2 u1 = BW == BW_ISO ? u0 : ld(&S.su[1][s]), u2 = BW == BW_ISO ? u0 : ld(&S.su[2][s]);
+        pair2(x.x, y.x, z.x, u0.x, u1.x, u2.x, c.x, a0, a1);
+        pair2(x.y, y.y, z.y, u0.y, u1.y, u2.y, c.y, a2, a3);
     };
     auto add = [&](float v) {  // compensated running sum (TwoSum)
         const float t = sum + v;
@@ -1986,22 +2036,24 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
             nl = warp_walk(a.e.tv, test, S.stack, spv, S.leaves, kBatch);
             if (nl == 0) break;
         }
+        seen += nl;
+        wide = seen >= kWideLeaves;
         // software pipeline: the next candidate leaf's point is loaded one step ahead
         float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 en = pn;
-        {
-            const int64_t j0 = (int64_t)S.leaves[0] * kLeaf + lane;
+        if (part < nl) {
+            const int64_t j0 = (int64_t)S.leaves[part] * kLeaf + lane;
             if (j0 < a.e.tv.n) {
                 pn = __ldg(&a.e.tv.pos[j0]);
                 if (BW == BW_ANISO) en = __ldg(&a.e.ell[j0]);
             }
         }
-        for (int li = 0; li < nl; ++li) {
+        for (int li = part; li < nl; li += SPLIT) {
             const int64_t j = (int64_t)S.leaves[li] * kLeaf + lane;
             const float4 p = pn;
             const float4 pe = en;
-            if (li + 1 < nl) {
-                const int64_t jn = (int64_t)S.leaves[li + 1] * kLeaf + lane;
+            if (li + SPLIT < nl) {
+                const int64_t jn = (int64_t)S.leaves[li + SPLIT] * kLeaf + lane;
                 if (jn < a.e.tv.n) {
                     pn = __ldg(&a.e.tv.pos[jn]);
                     if (BW == BW_ANISO) en = __ldg(&a.e.ell[jn]);
@@ -2031,6 +2083,15 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
                     qlb = fmaf(t, t, qlb);
                 }
                 ok = ok && qlb < KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
+                if (wide && ok) {
+                    ok = false;
+                    for (int e = 0; e < kLeaf; ++e) {
+                        const float4 w = S.q[e];
+                        const float tx = (w.x - p.x) * r[0], ty = (w.y - p.y) * r[1], tz = (w.z - p.z) * r[2];
+                        ok = ok || fmaf(tz, tz, fmaf(ty, ty, tx * tx)) <
+                                       KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
+                    }
+                }
             }
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok) {
@@ -2053,10 +2114,7 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
                 __syncwarp();
                 float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
-                for (int e = 0; e < kLeaf; e += 4) {
-                    pair2(head + e, a0, a1);
-                    pair2(head + e + 2, a2, a3);
-                }
+                for (int e = 0; e < kLeaf; e += 4) quad(head + e, a0, a1, a2, a3);
                 head ^= kLeaf;
                 cnt -= kLeaf;
                 add((a0 + a1) + (a2 + a3));
@@ -2065,23 +2123,30 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
         }
         nl = 0;
     }
-    // the staged remainder (cnt < 32 entries from head), padded to an even
-    // count with an entry of zero weight
-    if (cnt & 1) {
-        if (lane == 0) {
-            const int s = (head + cnt) & (kPtRing - 1);
-            S.sx[s] = S.sy[s] = S.sz[s] = S.sc[s] = 0.f;
-            S.su[0][s] = S.su[1][s] = S.su[2][s] = 0.f;
-        }
+    // the staged remainder (cnt < 32 entries from head), padded to a multiple of 4 with
+    // entries of zero weight
+    const int pad = (4 - (cnt & 3)) & 3;
+    if (lane < pad) {
+        const int s = (head + cnt + lane) & (kPtRing - 1);
+        S.sx[s] = S.sy[s] = S.sz[s] = S.sc[s] = 0.f;
+        S.su[0][s] = S.su[1][s] = S.su[2][s] = 0.f;
     }
     __syncwarp();
     if (cnt > 0) {
-        float a0 = 0.f, a1 = 0.f;
-        for (int e = 0; e < cnt; e += 2) pair2(head + e, a0, a1);
-        if (CNT && (cnt & 1)) --npairs;  // the padding entry is "in support" (q = 0)
-        add(a0 + a1);
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        for (int e = 0; e < cnt; e += 4) quad(head + e, a0, a1, a2, a3);
+        if (CNT) npairs -= (unsigned)pad;  // the padding entries are "in support" (q = 0)
+        add((a0 + a1) + (a2 + a3));
     }
-    if (active) a.rho_sorted[oi] = (float)(((double)sum + (double)cmp) * s_inv);
+    double total = (double)sum + (double)cmp;
+    if (SPLIT > 1) {
+        s_part[warp][lane] = total;
+        __syncthreads();
+        if (part != 0) return;
+#pragma unroll
+        for (int w = 1; w < SPLIT; ++w) total += s_part[warp + w][lane];
+    }
+    if (active) a.rho_sorted[oi] = (float)(total * s_inv);
     if (CNT) {
         if (!active) npairs = 0;
 #pragma unroll
@@ -2094,11 +2159,18 @@ template <int KER, int BW, bool CLIP>
 static cudaError_t launch_points(const PointsArgs &a, int64_t nleaf, cudaStream_t s) {
     if (a.pairs) {
         KTimer t("k_points_count", s);
-        return launch(k_points<KER, BW, CLIP, true>, dim3(blocks_for(nleaf, kPtWarps)),
+        return launch(k_points<KER, BW, CLIP, true, 1>, dim3(blocks_for(nleaf, kPtWarps)),
                       dim3(kPtWarps * 32), 0, s, a);
     }
     KTimer t("k_points", s);
-    return launch(k_points<KER, BW, CLIP, false>, dim3(blocks_for(nleaf, kPtWarps)),
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // below two waves of resident warps (32 an SM) a block shares each leaf
+    if (nleaf < (int64_t)sms * 64)
+        return launch(k_points<KER, BW, CLIP, false, kPtWarps>, dim3((unsigned)nleaf), dim3(kPtWarps * 32), 0, s, a);
+    return launch(k_points<KER, BW, CLIP, false, 1>, dim3(blocks_for(nleaf, kPtWarps)),
                   dim3(kPtWarps * 32), 0, s, a);
 }
 
