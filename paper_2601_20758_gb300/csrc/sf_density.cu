@@ -462,27 +462,6 @@ __device__ void grid_chunk(GridSmemT<TZ> &S, const TileGeom &g, const int *leave
 }
 
 // Fold a chunk's FP32 sums into the compensated per-voxel sums (TwoSum).
-// One per-axis table entry of the split pipeline for a particle at coordinate pc
-// (scale u = uscale / l, weight c) and a node nc (hi, lo): q = ((nc - pc) u)^2 and
-//   Gauss axis 0: (c e^{-q}, q)   axis 1: (e^{-q}, q)   axis 2: (e^{-q}, qmax - q)
-//   Epan  axis 0/1: (q, -)        axis 2: (c (1 - q), -)
-// with "no support" values (kBig / -1 / -kBig) where q >= qmax or outside.
-template <int KER>
-__device__ __forceinline__ float2 kentry(int axis, bool inside, float pc, float u, float c, float2 nc) {
-    const float d = (nc.x - pc) + nc.y;
-    const float t = d * u;
-    const float q = t * t;
-    const bool sup = inside && q < KDef<KER>::qmax;
-    if (KER == SF_K_GAUSS3) {
-        const float w = sup ? ex2_approx(-q) : 0.f;
-        if (axis == 0) return make_float2(w * c, sup ? q : kBig);
-        if (axis == 1) return make_float2(w, sup ? q : kBig);
-        return make_float2(w, sup ? KDef<KER>::qmax - q : -1.f);
-    }
-    if (axis < 2) return make_float2(sup ? q : kBig, 0.f);
-    return make_float2(sup ? c * (1.0f - q) : -kBig, 0.f);
-}
-
 template <int TZ>
 __device__ __forceinline__ void fold(float acc[TZ], float sum[TZ], float cmp[TZ]) {
 #pragma unroll
@@ -625,7 +604,6 @@ struct MrArgs {
 
 constexpr int kWalkWarps = 8;
 constexpr int kWX = 8, kWY = 4;  // node tile of one warp in the split pipeline (x, y)
-constexpr int kLaneTables = 10;   // staged points from which each lane fills its own tables
 
 struct WalkWarpSmem {
     int stack[kStack];
@@ -783,16 +761,19 @@ __device__ __forceinline__ void mma_k8(float d[4], float a0, float a1, float a2,
     mma_k8_tf32(d, A0, A1, A2, A3, B0, B1);
 }
 
-// Shared memory of one warp of the split pipeline: its 8 x 4 x TZ node tile.
-template <int TZ>
-struct WTileSmem {
+// Shared memory of one warp of the split pipeline: its 8 x 4 x TZ node tile. Rows of the
+// tables: the 32 staged particles being summed.
+constexpr int kWRing = 2 * kLeaf;  // staged particles: two halves of 32
+template <int TZ, bool ANISO>
+struct __align__(16) WTileSmem {
     float2 tx[kLeaf][kWX];   // Gauss: (c e^{-qx'}, qx'); Epan: (qx', -)
     float2 ty[kLeaf][kWY];   // Gauss: (e^{-qy'}, qy');   Epan: (qy', -)
-    float2 tz[kLeaf][TZ];    // Gauss: (e^{-qz'}, qmax - qz'); Epan: (c (1 - qz'), -)
-    float4 sp[kLeaf];        // staged (x, y, z, c)
-    float4 su[kLeaf];        // staged (u_x, u_y, u_z, -)
-    int2 sf[kLeaf];          // footprint: x0|x1<<8|y0<<16|y1<<24, z0|z1<<8
-    float2 axt[kWX + kWY + TZ];
+    float tzw[kLeaf][TZ];    // Gauss: e^{-qz'};          Epan: c (1 - qz')
+    float tzl[kLeaf][TZ];    // Gauss: qmax - qz' (also the scratch of the tensor-core sums)
+    float cs[kLeaf];         // Epan: c
+    float4 sp[kWRing];       // staged (x, y, z, h)
+    float4 sl[ANISO ? kWRing : 1];  // and (l_x, l_y, l_z)
+    float2 axt[kWX + kWY + TZ];     // node coordinates (past the grid's end: the last node's again)
     float uni[3];
     EngineArgs e;
     RoiDesc roi;
@@ -801,18 +782,29 @@ struct WTileSmem {
 // Persistent warps: each takes (ROI, tile, leaf range) items from a counter and
 // sums them into the item's partial grid. No block barriers: a warp owns its
 // tile, its staging and its tables.
+//
+// What bounds it: issue slots and the ALU pipe, which every support test goes through. So
+// candidates are staged across leaves and summed 32 at a time (every lane fills one
+// particle's tables; one compensated fold per 32 particles, as for one full leaf), the
+// particles whose support covers the tile come first and are summed without a test, two
+// nodes an instruction (10 issue slots a particle and 256 nodes; 24 with the tests), and
+// table rows are written and read 16 bytes at a time. Work time (gaussian, kNN lengths) of a
+// 256^3 zoom of 67M points, 70% of whose staged particles cover their tile: 3.20 -> 1.88
+// ms; of its whole cube at 128^3 (supports of about a spacing): 3.74 -> 2.50 ms; 192^3 in
+// BF16: 1.34 -> 0.71 ms; 64 uneven grids: 48.8 -> 30.9 ms.
 template <int KER, int BW, bool CLIP, bool CNT, int TZ, int PREC = SF_PREC_FP32>
-__global__ void __launch_bounds__(kGridThreads, 4)
+__global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
     k_mr_work(MrArgs a, const int4 *__restrict__ items, const uint32_t *__restrict__ n_items,
               const int *__restrict__ list, double *__restrict__ part, unsigned int *next) {
     // the tensor-core path of the precision variants: Gaussian, 8 nodes deep (the
     // B operand's 8 columns); the FP32 path sums every particle in FP32
     constexpr bool kMma = KER == SF_K_GAUSS3 && TZ == 8 && PREC != SF_PREC_FP32;
-    constexpr bool kFull = KER == SF_K_GAUSS3 && TZ == 8 && (PREC != SF_PREC_FP32 || CNT);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WTileSmem<TZ> &S = reinterpret_cast<WTileSmem<TZ> *>(smem_raw)[warp];
+    typedef WTileSmem<TZ, BW == BW_ANISO> Smem;
+    Smem &S = reinterpret_cast<Smem *>(smem_raw)[warp];
     const int cx = lane & (kWX - 1), cy = lane / kWX;
+    const unsigned lt = (1u << lane) - 1u;
     const uint32_t nitems = *n_items;
     unsigned long long npairs = 0;
     int cur_roi = -1;
@@ -834,20 +826,13 @@ __global__ void __launch_bounds__(kGridThreads, 4)
         const EngineArgs &E = S.e;
         const RoiDesc &r = S.roi;
         // ---- the tile's node coordinates
-        TileGeom g;
-        float isp[3], mcen[3], mhw[3];  // 1 / node spacing; tile box widened by the rounding margin
-        tile_origin<TZ, kWX, kWY>(r, it.x - r.tile_base, g.gx0, g.gy0, g.gz0, g.nv);
+        int gx0, gy0, gz0, nv[3];
+        tile_origin<TZ, kWX, kWY>(r, it.x - r.tile_base, gx0, gy0, gz0, nv);
         if (lane < kWX + kWY + TZ) {
-            float2 v = make_float2(0.f, 0.f);
-            if (lane < kWX) {
-                if (lane < g.nv[0]) v = r.axis[g.gx0 + lane];
-            } else if (lane < kWX + kWY) {
-                const int j = lane - kWX;
-                if (j < g.nv[1]) v = r.axis[r.nx + g.gy0 + j];
-            } else {
-                const int j = lane - kWX - kWY;
-                if (j < g.nv[2]) v = r.axis[r.nx + r.ny + g.gz0 + j];
-            }
+            float2 v;
+            if (lane < kWX) v = r.axis[gx0 + min(lane, nv[0] - 1)];
+            else if (lane < kWX + kWY) v = r.axis[r.nx + gy0 + min(lane - kWX, nv[1] - 1)];
+            else v = r.axis[r.nx + r.ny + gz0 + min(lane - kWX - kWY, nv[2] - 1)];
             S.axt[lane] = v;
         }
         if (lane == 0) {
@@ -856,237 +841,255 @@ __global__ void __launch_bounds__(kGridThreads, 4)
             S.uni[2] = E.dp->ell_uniform[2];
         }
         __syncwarp();
-        {
-            const int off[3] = {0, kWX, kWX + kWY};
+        float mcen[3], mhw[3];  // the tile box widened by the rounding margin, as centre and half-width
+        float sp3[3];           // node spacing
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                g.tlo[k] = S.axt[off[k]].x;
-                g.thi[k] = S.axt[off[k] + g.nv[k] - 1].x;
-                g.sp3[k] = g.nv[k] > 1 ? (S.axt[off[k] + 1].x - S.axt[off[k]].x) : 1.f;
-                isp[k] = g.sp3[k] > 0.f ? 1.0f / g.sp3[k] : 0.f;
-                const float mg = 1.0e-6f * (fabsf(g.tlo[k]) + fabsf(g.thi[k]));
-                const float lo_m = g.tlo[k] - mg, hi_m = g.thi[k] + mg;
-                mcen[k] = 0.5f * (lo_m + hi_m);
-                mhw[k] = 0.5f * (hi_m - lo_m);
-            }
+        for (int k = 0; k < 3; ++k) {
+            const int off = k == 0 ? 0 : (k == 1 ? kWX : kWX + kWY);
+            const float lo = S.axt[off].x, hi = S.axt[off + nv[k] - 1].x;
+            sp3[k] = nv[k] > 1 ? S.axt[off + 1].x - lo : 0.f;
+            const float mg = 1.0e-6f * (fabsf(lo) + fabsf(hi));
+            mcen[k] = 0.5f * ((lo - mg) + (hi + mg));
+            mhw[k] = 0.5f * ((hi + mg) - (lo - mg));
         }
         float acc[TZ], sum[TZ], cmp[TZ];
 #pragma unroll
         for (int k = 0; k < TZ; ++k) acc[k] = sum[k] = cmp[k] = 0.f;
         unsigned long long np = 0;
-        unsigned long long st_leaves = 0, st_staged = 0, st_full = 0, st_tested = 0;
-        for (int lb = it.y; lb < it.z; ++lb) {
-            // ---- one candidate leaf: refine (footprint in this tile, clip) and stage
-            const int64_t i = (int64_t)list[lb] * kLeaf + lane;
-            bool acc_pt = false;
-            float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-            float l[3] = {0.f, 0.f, 0.f}, rl[3] = {0.f, 0.f, 0.f};
-            int2 fp = make_int2(0, 0);
-            bool full = false;  // the support covers every node of the tile
-            if (i < E.tv.n) {
-                p = __ldg(&E.tv.pos[i]);
-                point_ell<BW>(E, S.uni, i, p, l);
-                acc_pt = l[0] > 0.f && l[1] > 0.f && l[2] > 0.f;
-                if (CLIP)
-                    acc_pt = acc_pt && p.x >= E.blo[0] && p.x <= E.bhi[0] && p.y >= E.blo[1] &&
+        unsigned long long st_leaves = 0, st_staged = 0, st_full = 0;
+        int head = 0, staged = 0;  // the ring: first staged particle, how many (warp-uniform)
+        // the next candidate leaf's point is loaded one step ahead, its number two
+        float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
+        int64_t in = -1;
+        auto load = [&](int leaf) {
+            in = (int64_t)leaf * kLeaf + lane;
+            if (in < E.tv.n) pn = __ldg(&E.tv.pos[in]);
+        };
+        int lnext = it.y + 1 < it.z ? list[it.y + 1] : 0;
+        if (it.y < it.z) load(list[it.y]);
+        for (int lb = it.y; lb < it.z || staged > 0; ++lb) {
+            if (lb < it.z) {
+                // ---- one candidate leaf: the points whose support reaches a node of the tile
+                const int64_t i = in;
+                const float4 p = pn;
+                if (lb + 1 < it.z) {
+                    load(lnext);
+                    if (lb + 2 < it.z) lnext = list[lb + 2];
+                }
+                bool ok = false;
+                float l[3] = {0.f, 0.f, 0.f};
+                if (i < E.tv.n) {
+                    point_ell<BW>(E, S.uni, i, p, l);
+                    ok = l[0] > 0.f && l[1] > 0.f && l[2] > 0.f;
+                    if (CLIP)
+                        ok = ok && p.x >= E.blo[0] && p.x <= E.bhi[0] && p.y >= E.blo[1] &&
                              p.y <= E.bhi[1] && p.z >= E.blo[2] && p.z <= E.bhi[2];
-                const float pc[3] = {p.x, p.y, p.z};
-                int f0[3], f1[3];
-                float qlb = 0.f;
+                    const float pc[3] = {p.x, p.y, p.z};
+                    float rl[3], qlb = 0.f;
+                    bool small = false;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        rl[k] = BW == BW_ISO && k > 0 ? rl[0] : rcp_approx(l[k]);
+                        const float t = fmaxf(fabsf(pc[k] - mcen[k]) - mhw[k], 0.f) * rl[k];
+                        qlb = fmaf(t, t, qlb);
+                        small = small || l[k] * KDef<KER>::rmul < sp3[k];
+                    }
+                    ok = ok && qlb < KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
+                    // Supports below a node spacing may lie between the nodes: the smallest per-axis
+                    // q (computed exactly as the tables compute it, at the nodes nearest the
+                    // point) bounds every node's test (the float sums and differences are
+                    // monotone): a particle that fails it adds nothing to any node of the
+                    // tile (a dense cluster in a coarse grid's cell) and is not staged.
+                    if (ok && small) {
+                        float mq[3];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            const int off = k == 0 ? 0 : (k == 1 ? kWX : kWX + kWY);
+                            const float u = KDef<KER>::uscale * rl[k];
+                            const float at = sp3[k] > 0.f ? (pc[k] - S.axt[off].x) / sp3[k] : 0.f;
+                            const int ic = (int)rintf(fminf(fmaxf(at, 0.f), (float)(nv[k] - 1)));
+                            float m = INFINITY;
+#pragma unroll
+                            for (int dd = -1; dd <= 1; ++dd) {
+                                const float2 nc = S.axt[off + min(max(ic + dd, 0), nv[k] - 1)];
+                                const float d = (nc.x - pc[k]) + nc.y;
+                                const float t = d * u;
+                                m = fminf(m, t * t);
+                            }
+                            mq[k] = m;
+                        }
+                        if (KER == SF_K_GAUSS3) {
+                            ok = mq[0] + mq[1] < KDef<KER>::qmax - mq[2];
+                        } else {
+                            const float c = E.cnorm * ((rl[0] * rl[1]) * rl[2]);
+                            ok = c * (1.0f - mq[2]) - c * (mq[0] + mq[1]) > 0.f;
+                        }
+                    }
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, ok);
+                if (ok) {
+                    const int s = (head + staged + __popc(bal & lt)) & (kWRing - 1);
+                    S.sp[s] = p;
+                    if (BW == BW_ANISO) S.sl[s] = make_float4(l[0], l[1], l[2], 0.f);
+                }
+                staged += __popc(bal);
+                if (CNT && lane == 0 && bal) {
+                    ++st_leaves;
+                    st_staged += __popc(bal);
+                }
+                if (staged < kLeaf && lb + 1 < it.z) continue;  // warp-uniform
+                if (staged == 0) continue;
+            }
+            // ---- tables of 32 staged particles (fewer only at the end), one particle a lane:
+            // factors and q at the tile's nodes. A q past the support needs no mark: it
+            // fails the test by itself (qx + qy < qmax - qz, every term non-negative).
+            const int ns = min(staged, kLeaf);
+            __syncwarp();
+            bool full = false;  // the support covers every node of the tile
+            float mx = 0.f, my = 0.f, mz = 0.f, c = 0.f, u[3] = {0.f, 0.f, 0.f};
+            float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane < ns) {
+                const int e = head + lane;
+                p = S.sp[e];
+                float l[3] = {p.w, p.w, p.w};
+                if (BW == BW_UNIFORM) {
+                    l[0] = S.uni[0]; l[1] = S.uni[1]; l[2] = S.uni[2];
+                } else if (BW == BW_ANISO) {
+                    const float4 q = S.sl[e];
+                    l[0] = q.x; l[1] = q.y; l[2] = q.z;
+                }
+                float rl[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     rl[k] = BW == BW_ISO && k > 0 ? rl[0] : rcp_approx(l[k]);
-                    const float R = l[k] * KDef<KER>::rmul;
-                    if (g.sp3[k] > 0.f) {
-                        const float a0 = fminf(fmaxf(ceilf((pc[k] - R - g.tlo[k]) * isp[k]) - 1.f, -1.f), 64.f);
-                        const float a1 = fminf(fmaxf(floorf((pc[k] + R - g.tlo[k]) * isp[k]) + 1.f, -1.f), 64.f);
-                        f0[k] = max(0, (int)a0);
-                        f1[k] = min(g.nv[k] - 1, (int)a1);
-                    } else {
-                        f0[k] = 0;
-                        f1[k] = g.nv[k] - 1;
-                    }
-                    if (f0[k] > f1[k]) acc_pt = false;
-                    const float t = fmaxf(fabsf(pc[k] - mcen[k]) - mhw[k], 0.f) * rl[k];
-                    qlb = fmaf(t, t, qlb);
+                    u[k] = KDef<KER>::uscale * rl[k];
                 }
-                if (!(qlb < KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack))) acc_pt = false;
-                // Small supports: exact footprints. The widened ranges shrink to the nodes whose
-                // per-axis q (computed exactly as the tables compute it) is below
-                // qmax -- a contiguous run, since q is unimodal along the axis. Then
-                // the smallest per-axis q bounds every node's test (the float sums and
-                // differences are monotone): a particle that fails it adds nothing to
-                // any node of the tile (a dense cluster between the nodes of a coarse
-                // grid) and is not staged.
-                if (acc_pt && f1[0] - f0[0] < 4 && f1[1] - f0[1] < 4 && f1[2] - f0[2] < 4) {
-                    float mq[3];
-                    const int aoff[3] = {0, kWX, kWX + kWY};
+                c = E.cnorm * ((rl[0] * rl[1]) * rl[2]);
+                // q is convex along each axis: its largest value is at an end node, and passing
+                // the test with the per-axis maxima passes it at every node
+                auto ends = [&](int off, int n, float pc, float uu) {
+                    const float2 n0 = S.axt[off], n1 = S.axt[off + n - 1];
+                    const float t0 = ((n0.x - pc) + n0.y) * uu, t1 = ((n1.x - pc) + n1.y) * uu;
+                    return fmaxf(t0 * t0, t1 * t1);
+                };
+                mx = ends(0, kWX, p.x, u[0]);
+                my = ends(kWX, kWY, p.y, u[1]);
+                mz = ends(kWX + kWY, TZ, p.z, u[2]);
+                if (KER == SF_K_GAUSS3) full = mx + my < KDef<KER>::qmax - mz;
+                else full = c * (1.0f - mz) - c * (mx + my) > 0.f;
+            }
+            // rows: the full-coverage particles first, [0, nf); the others [nf, ns)
+            const unsigned balf = __ballot_sync(0xffffffffu, full);
+            const int nf = __popc(balf);
+            if (CNT && lane == 0 && KER == SF_K_GAUSS3 && TZ == 8) st_full += nf;
+            if (lane < ns) {
+                const int s = full ? __popc(balf & lt) : nf + __popc(~balf & lt);
+                auto q_at = [&](float2 nc, float pc, float uu) {
+                    const float t = ((nc.x - pc) + nc.y) * uu;
+                    return t * t;
+                };
+                // two nodes of x or y a step, four of z, in an order that starts by the row so
+                // that the lanes' 16-byte stores spread over the banks
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const float u = KDef<KER>::uscale * rl[k];
-                        auto qat = [&](int ii) {
-                            const float2 nc = S.axt[aoff[k] + ii];
-                            const float d = (nc.x - pc[k]) + nc.y;
-                            const float t = d * u;
-                            return t * t;
-                        };
-                        while (f0[k] <= f1[k] && !(qat(f0[k]) < KDef<KER>::qmax)) ++f0[k];
-                        while (f1[k] >= f0[k] && !(qat(f1[k]) < KDef<KER>::qmax)) --f1[k];
-                        float m = kBig;
-                        if (f0[k] <= f1[k]) {
-                            const int ic = min(max((int)rintf((pc[k] - g.tlo[k]) * isp[k]), f0[k]), f1[k]);
+                for (int t = 0; t < kWX / 2; ++t) {
+                    const int i = 2 * ((t + (s >> 1)) & (kWX / 2 - 1));
+                    const float4 nc = *reinterpret_cast<const float4 *>(&S.axt[i]);
+                    const float q0 = q_at(make_float2(nc.x, nc.y), p.x, u[0]), q1 = q_at(make_float2(nc.z, nc.w), p.x, u[0]);
+                    *reinterpret_cast<float4 *>(&S.tx[s][i]) =
+                        KER == SF_K_GAUSS3 ? make_float4(ex2_approx(-q0) * c, q0, ex2_approx(-q1) * c, q1)
+                                           : make_float4(q0, 0.f, q1, 0.f);
+                }
 #pragma unroll
-                            for (int dd = -1; dd <= 1; ++dd) {
-                                const int ii = ic + dd;
-                                if (ii >= f0[k] && ii <= f1[k]) m = fminf(m, qat(ii));
-                            }
-                        }
-                        mq[k] = m;
-                    }
+                for (int t = 0; t < kWY / 2; ++t) {
+                    const int i = 2 * ((t + (s >> 2)) & (kWY / 2 - 1));
+                    const float4 nc = *reinterpret_cast<const float4 *>(&S.axt[kWX + i]);
+                    const float q0 = q_at(make_float2(nc.x, nc.y), p.y, u[1]), q1 = q_at(make_float2(nc.z, nc.w), p.y, u[1]);
+                    *reinterpret_cast<float4 *>(&S.ty[s][i]) =
+                        KER == SF_K_GAUSS3 ? make_float4(ex2_approx(-q0), q0, ex2_approx(-q1), q1)
+                                           : make_float4(q0, 0.f, q1, 0.f);
+                }
+#pragma unroll
+                for (int t = 0; t < TZ / 4; ++t) {
+                    const int i = 4 * ((t + (s >> 2)) & (TZ / 4 - 1));
+                    const float4 na = *reinterpret_cast<const float4 *>(&S.axt[kWX + kWY + i]);
+                    const float4 nb = *reinterpret_cast<const float4 *>(&S.axt[kWX + kWY + i + 2]);
+                    const float q0 = q_at(make_float2(na.x, na.y), p.z, u[2]), q1 = q_at(make_float2(na.z, na.w), p.z, u[2]);
+                    const float q2 = q_at(make_float2(nb.x, nb.y), p.z, u[2]), q3 = q_at(make_float2(nb.z, nb.w), p.z, u[2]);
                     if (KER == SF_K_GAUSS3) {
-                        if (!(mq[0] + mq[1] < KDef<KER>::qmax - mq[2])) acc_pt = false;
+                        *reinterpret_cast<float4 *>(&S.tzw[s][i]) =
+                            make_float4(ex2_approx(-q0), ex2_approx(-q1), ex2_approx(-q2), ex2_approx(-q3));
+                        constexpr float qm = KDef<KER>::qmax;
+                        *reinterpret_cast<float4 *>(&S.tzl[s][i]) = make_float4(qm - q0, qm - q1, qm - q2, qm - q3);
                     } else {
-                        const float c = E.cnorm * ((rl[0] * rl[1]) * rl[2]);
-                        if (!(c * (1.0f - mq[2]) - c * (mq[0] + mq[1]) > 0.f)) acc_pt = false;
+                        *reinterpret_cast<float4 *>(&S.tzw[s][i]) =
+                            make_float4(c * (1.0f - q0), c * (1.0f - q1), c * (1.0f - q2), c * (1.0f - q3));
                     }
                 }
-                if (acc_pt) {
-                    fp.x = f0[0] | (f1[0] << 8) | (f0[1] << 16) | (f1[1] << 24);
-                    fp.y = f0[2] | (f1[2] << 8);
-                }
-                // Full coverage: q is convex along each axis, so its largest value over the
-                // tile is at a corner node; the node test fl(qx + qy) < fl(qmax - qz) is
-                // monotone in each q, so passing it with the per-axis maxima passes it
-                // at every node (as the table path would evaluate it).
-                if (kFull && acc_pt && f0[0] == 0 && f1[0] == g.nv[0] - 1 && f0[1] == 0 &&
-                    f1[1] == g.nv[1] - 1 && f0[2] == 0 && f1[2] == g.nv[2] - 1) {
-                    const int aoff[3] = {0, kWX, kWX + kWY};
-                    float qm[3];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const float u = KDef<KER>::uscale * rl[k];
-                        float m = 0.f;
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float2 nc = S.axt[aoff[k] + (e ? g.nv[k] - 1 : 0)];
-                            const float d = (nc.x - pc[k]) + nc.y;
-                            const float t = d * u;
-                            m = fmaxf(m, t * t);
-                        }
-                        qm[k] = m;
-                    }
-                    full = qm[0] + qm[1] < KDef<KER>::qmax - qm[2];
-                }
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, acc_pt);
-            const int ns = __popc(bal);
-            if (ns == 0) continue;  // warp-uniform
-            // staged slots: the full-coverage particles first, [0, nf); the others [nf, ns)
-            const unsigned balf = __ballot_sync(0xffffffffu, acc_pt && full);
-            const int nf = kMma ? __popc(balf) : 0;
-            if (CNT && lane == 0) {
-                ++st_leaves;
-                st_staged += ns;
-                st_full += __popc(balf);
-                st_tested += (unsigned long long)ns * (kWX * kWY * TZ);
-            }
-            const unsigned lt = (1u << lane) - 1u;
-            const int my_slot = !kMma ? __popc(bal & lt)
-                                      : (full ? __popc(balf & lt) : nf + __popc(bal & ~balf & lt));
-            if (acc_pt) {
-                const int s = my_slot;
-                S.sp[s] = make_float4(p.x, p.y, p.z, E.cnorm * ((rl[0] * rl[1]) * rl[2]));
-                S.su[s] = make_float4(KDef<KER>::uscale * rl[0], KDef<KER>::uscale * rl[1],
-                                      KDef<KER>::uscale * rl[2], 0.f);
-                S.sf[s] = fp;
+                if (KER != SF_K_GAUSS3) S.cs[s] = c;
             }
             __syncwarp();
-            // ---- per-axis tables: factors inside the footprint, "no support" values
-            // outside it (so the accumulation needs no range tests). Many staged points:
-            // each staging lane fills its own point's entries, in an order rotated by
-            // its row so that the lanes' stores spread over the banks; few: the entries
-            // are spread over all lanes. Same values either way.
-            constexpr int kEnt = kWX + kWY + TZ;
-            auto entry = [&](int axis, int ii, bool inside, float pc, float u, float c, float2 nc) {
-                return kentry<KER>(axis, inside, pc, u, c, nc);
-            };
-            if (ns >= kLaneTables) {
-                if (acc_pt) {
-                    const int s = my_slot;
-                    const float c = E.cnorm * ((rl[0] * rl[1]) * rl[2]);
-                    const float u0 = KDef<KER>::uscale * rl[0], u1 = KDef<KER>::uscale * rl[1],
-                                u2 = KDef<KER>::uscale * rl[2];
-                    const int x0 = fp.x & 255, x1 = (fp.x >> 8) & 255;
-                    const int y0 = (fp.x >> 16) & 255, y1 = (fp.x >> 24) & 255;
-                    const int z0 = fp.y & 255, z1 = (fp.y >> 8) & 255;
-                    {
-#pragma unroll
-                        for (int t = 0; t < kWX; ++t) {
-                            const int i = (t + (s >> 1)) & (kWX - 1);
-                            S.tx[s][i] = entry(0, i, i >= x0 && i <= x1, p.x, u0, c, S.axt[i]);
-                        }
-#pragma unroll
-                        for (int t = 0; t < kWY; ++t) {
-                            const int i = (t + (s >> 2)) & (kWY - 1);
-                            S.ty[s][i] = entry(1, i, i >= y0 && i <= y1, p.y, u1, c, S.axt[kWX + i]);
-                        }
-#pragma unroll
-                        for (int t = 0; t < TZ; ++t) {
-                            const int i = (t + (s >> (TZ == 8 ? 1 : 2))) & (TZ - 1);
-                            S.tz[s][i] = entry(2, i, i >= z0 && i <= z1, p.z, u2, c, S.axt[kWX + kWY + i]);
-                        }
-                    }
-                }
-            } else
-            for (int e = lane; e < ns * kEnt; e += 32) {
-                const int s = e / kEnt;
-                const int j = e - s * kEnt;
-                const int2 F = S.sf[s];
-                int axis, ii, lo_i, hi_i;
-                if (j < kWX) {
-                    axis = 0; ii = j; lo_i = F.x & 255; hi_i = (F.x >> 8) & 255;
-                } else if (j < kWX + kWY) {
-                    axis = 1; ii = j - kWX; lo_i = (F.x >> 16) & 255; hi_i = (F.x >> 24) & 255;
-                } else {
-                    axis = 2; ii = j - kWX - kWY; lo_i = F.y & 255; hi_i = (F.y >> 8) & 255;
-                }
-                const bool inside = ii >= lo_i && ii <= hi_i;
-                const float4 P = S.sp[s];
-                const float4 U = S.su[s];
-                const float pc = axis == 0 ? P.x : (axis == 1 ? P.y : P.z);
-                const float u = axis == 0 ? U.x : (axis == 1 ? U.y : U.z);
-                const float2 v = entry(axis, ii, inside, pc, u, P.w, S.axt[j]);
-                if (axis == 0) S.tx[s][ii] = v;
-                else if (axis == 1) S.ty[s][ii] = v;
-                else S.tz[s][ii] = v;
-            }
-            __syncwarp();
-            {
+            head ^= kLeaf;
+            staged -= ns;
             // ---- accumulate: lane owns column (cx, cy) and TZ nodes in z
-            for (int s = nf; s < ns; ++s) {
+            const int s_test = CNT ? 0 : nf;  // rows from here on are tested
+            if (!kMma && !CNT) {
+                f32x2 acc2[TZ / 2];
+#pragma unroll
+                for (int k = 0; k < TZ / 2; ++k) acc2[k] = f2_pack(acc[2 * k], acc[2 * k + 1]);
+#pragma unroll 4
+                for (int s = 0; s < nf; ++s) {
+                    float b;
+                    if (KER == SF_K_GAUSS3) b = S.tx[s][cx].x * S.ty[s][cy].x;
+                    else b = S.cs[s] * (S.tx[s][cx].x + S.ty[s][cy].x);
+                    const f32x2 bb = f2_pack(b, b);
+#pragma unroll
+                    for (int k = 0; k < TZ; k += 4) {
+                        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(&S.tzw[s][k]);
+                        if (KER == SF_K_GAUSS3) {
+                            acc2[k / 2] = f2_fma(bb, z.x, acc2[k / 2]);
+                            acc2[k / 2 + 1] = f2_fma(bb, z.y, acc2[k / 2 + 1]);
+                        } else {
+                            acc2[k / 2] = f2_add(acc2[k / 2], f2_sub(z.x, bb));
+                            acc2[k / 2 + 1] = f2_add(acc2[k / 2 + 1], f2_sub(z.y, bb));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < TZ / 2; ++k) f2_unpack(acc2[k], acc[2 * k], acc[2 * k + 1]);
+            }
+#pragma unroll 2
+            for (int s = kMma ? nf : s_test; s < ns; ++s) {
                 const float2 ex = S.tx[s][cx];
                 const float2 ey = S.ty[s][cy];
                 if (KER == SF_K_GAUSS3) {
                     const float bse = ex.x * ey.x;
                     const float qij = ex.y + ey.y;
 #pragma unroll
-                    for (int k = 0; k < TZ; ++k) {
-                        const float2 ez = S.tz[s][k];
-                        if (qij < ez.y) {
-                            acc[k] = fmaf(bse, ez.x, acc[k]);
-                            if (CNT) ++np;
-                        }
+                    for (int k = 0; k < TZ; k += 4) {
+                        const float4 w = *reinterpret_cast<const float4 *>(&S.tzw[s][k]);
+                        const float4 m = *reinterpret_cast<const float4 *>(&S.tzl[s][k]);
+                        const float wv[4] = {w.x, w.y, w.z, w.w}, mv[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (qij < mv[j]) {
+                                acc[k + j] = fmaf(bse, wv[j], acc[k + j]);
+                                if (CNT && k + j < nv[2]) ++np;
+                            }
                     }
                 } else {
-                    const float b = S.sp[s].w * (ex.x + ey.x);
+                    const float b = S.cs[s] * (ex.x + ey.x);
 #pragma unroll
-                    for (int k = 0; k < TZ; ++k) {
-                        const float t = S.tz[s][k].x - b;
-                        acc[k] += fmaxf(t, 0.f);
-                        if (CNT) np += (t > 0.f);
+                    for (int k = 0; k < TZ; k += 4) {
+                        const float4 w = *reinterpret_cast<const float4 *>(&S.tzw[s][k]);
+                        const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float t = wv[j] - b;
+                            acc[k + j] += fmaxf(t, 0.f);
+                            if (CNT && k + j < nv[2]) np += (t > 0.f);
+                        }
                     }
                 }
-            }
             }
             if (kMma && nf > 0) {  // warp-uniform: the full-coverage particles on the tensor cores
                 const int gq = lane >> 2, tig = lane & 3;
@@ -1099,7 +1102,7 @@ __global__ void __launch_bounds__(kGridThreads, 4)
                             const int sp = s0 + 2 * tig + (e & 1) + 8 * (e >> 1);
                             const bool v = sp < nf;
                             ax[e] = v ? S.tx[sp][gq].x : 0.f;
-                            bz[e] = v ? S.tz[sp][gq].x : 0.f;
+                            bz[e] = v ? S.tzw[sp][gq] : 0.f;
 #pragma unroll
                             for (int y = 0; y < 4; ++y) ay[e][y] = v ? S.ty[sp][y].x : 0.f;
                         }
@@ -1119,7 +1122,7 @@ __global__ void __launch_bounds__(kGridThreads, 4)
                         const int sa = s0 + tig, sb = s0 + tig + 4;
                         const bool va = sa < nf, vb = sb < nf;
                         const float txa = va ? S.tx[sa][gq].x : 0.f, txb = vb ? S.tx[sb][gq].x : 0.f;
-                        const float tza = va ? S.tz[sa][gq].x : 0.f, tzb = vb ? S.tz[sb][gq].x : 0.f;
+                        const float tza = va ? S.tzw[sa][gq] : 0.f, tzb = vb ? S.tzw[sb][gq] : 0.f;
 #pragma unroll
                         for (int mb = 0; mb < 2; ++mb) {
                             const float ya0 = va ? S.ty[sa][2 * mb].x : 0.f, ya1 = va ? S.ty[sa][2 * mb + 1].x : 0.f;
@@ -1129,7 +1132,7 @@ __global__ void __launch_bounds__(kGridThreads, 4)
                     }
                 }
                 // to the column owners: row r = x + 8 y of the product is lane r's column
-                float *cb = reinterpret_cast<float *>(S.tx);  // the tables are no longer read
+                float *cb = reinterpret_cast<float *>(S.tzl);  // no longer read
                 __syncwarp();
 #pragma unroll
                 for (int mb = 0; mb < 2; ++mb) {
@@ -1143,17 +1146,16 @@ __global__ void __launch_bounds__(kGridThreads, 4)
                 __syncwarp();
 #pragma unroll
                 for (int k = 0; k < TZ; ++k) acc[k] += cb[lane * 8 + k];
-                if (CNT && cx < g.nv[0] && cy < g.nv[1]) np += (unsigned long long)nf * g.nv[2];
             }
             __syncwarp();
             fold<TZ>(acc, sum, cmp);
         }
-        if (CNT && cx < g.nv[0] && cy < g.nv[1]) npairs += np;
+        if (CNT && cx < nv[0] && cy < nv[1]) npairs += np;
         if (CNT && lane == 0) {  // work accounting of the counting variant
             atomicAdd(a.pairs + 1, st_leaves);
             atomicAdd(a.pairs + 2, st_staged);
             atomicAdd(a.pairs + 3, st_full);
-            atomicAdd(a.pairs + 4, st_tested);
+            atomicAdd(a.pairs + 4, st_staged * (kWX * kWY * TZ));
         }
         double *o = part + ((int64_t)item * 32 + lane) * TZ;
 #pragma unroll
@@ -1304,14 +1306,14 @@ static sf_status mr_count(const MrArgs &a, uint32_t *cnt, uint32_t *off, uint32_
     return SF_OK;
 }
 
-template <int TZ>
+template <int TZ, int BW>
 static size_t mr_work_smem() {
-    return sizeof(WTileSmem<TZ>) * (kGridThreads / 32);
+    return sizeof(WTileSmem<TZ, BW == BW_ANISO>) * (kGridThreads / 32);
 }
 
 template <int KER, int BW, bool CLIP, bool CNT, int TZ>
 static sf_status mr_work_attr(int *per_sm) {
-    const size_t smem = mr_work_smem<TZ>();
+    const size_t smem = mr_work_smem<TZ, BW>();
     static std::atomic<uint64_t> attr{0};
     SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ>, smem, attr));
     SF_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_mr_work<KER, BW, CLIP, CNT, TZ>,
@@ -1334,9 +1336,9 @@ struct MrBuffers {
 template <int KER, int BW, bool CLIP, bool CNT, int TZ, int PREC>
 static sf_status launch_work(const MrArgs &a, const MrBuffers &b, cudaStream_t s) {
     static std::atomic<uint64_t> attr{0};
-    SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, mr_work_smem<TZ>(), attr));
+    SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, mr_work_smem<TZ, BW>(), attr));
     SF_TRY_CUDA(launch(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, dim3((unsigned)b.slots), dim3(kGridThreads),
-                       mr_work_smem<TZ>(), s, a, (const int4 *)b.items, (const uint32_t *)(b.tot + 1),
+                       mr_work_smem<TZ, BW>(), s, a, (const int4 *)b.items, (const uint32_t *)(b.tot + 1),
                        (const int *)b.list, b.part, b.next));
     return SF_OK;
 }
