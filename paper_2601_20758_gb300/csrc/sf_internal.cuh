@@ -274,6 +274,9 @@ sf_status scan_u32(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint32_t *d
 // Result ends in (keys, vals); keys_tmp / vals_tmp are n-element scratch.
 sf_status radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *keys_tmp,
                            uint32_t *vals_tmp, int64_t n, int bits, cudaStream_t s);
+// Keys per block (the sort's count table holds 256 words per block).
+constexpr int64_t kRsTile1024 = 2 * 152 * 1024, kRsTile4096 = 2 * 152 * 4096;  // from how many keys on
+int64_t radix_sort_tile(int64_t n);
 // Order-preserving map of float bits to uint32 (total order on non-NaN floats).
 __host__ __device__ inline uint32_t float_to_ordered(float f) {
 #ifdef __CUDA_ARCH__

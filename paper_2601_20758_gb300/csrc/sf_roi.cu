@@ -205,8 +205,12 @@ static int64_t compact_peak(int64_t np, int64_t m) {
     int64_t peak = base + scan_parts_bytes(np);
     if (m > 0) {
         const int64_t pairs = 2 * scratch_round(8 * m) + 2 * scratch_round(4 * m);
-        const int64_t counts = scratch_round(4 * 256 * ((m + 4095) / 4096));
-        peak = std::max(peak, base + pairs + counts + scan_parts_bytes(256 * ((m + 4095) / 4096)));
+        // the sort's count table is not monotone in the points (few are sorted in small tiles):
+        // the largest for any number of points up to m
+        auto blocks = [](int64_t k) { return (k + radix_sort_tile(k) - 1) / radix_sort_tile(k); };
+        const int64_t nb = std::max(blocks(m), std::max(blocks(std::min<int64_t>(m, kRsTile1024 - 1)),
+                                                        blocks(std::min<int64_t>(m, kRsTile4096 - 1))));
+        peak = std::max(peak, base + pairs + scratch_round(4 * 256 * nb) + scan_parts_bytes(256 * nb));
     }
     return peak;
 }
