@@ -33,18 +33,62 @@ sf_status interp_points(sf_index *idx, const sf_box &roi, const GridSpec &g, con
                         cudaStream_t s, int tet);
 
 // Count the points of the scope and set N_eff (device); EMPTY_ROI is recorded
-// in the status word when the clip scope holds no point.
-__global__ void k_count_box(const float4 *__restrict__ pos, int64_t n, float3 lo, float3 hi,
-                            unsigned long long *cnt) {
-    unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 p = pos[i];
-        c += (p.x >= lo.x && p.x <= hi.x && p.y >= lo.y && p.y <= hi.y && p.z >= lo.z && p.z <= hi.z);
+// in the status word when the clip scope holds no point. One warp per quarter (8 leaves) of
+// a level-1 node: a node or leaf inside the box counts whole, one outside not at all, only the leaves that
+// cut its faces are read. (Reading every point took 51 us at 16.8M points, with the
+// cloud's size.)
+constexpr int kCountWarps = 8;
+__global__ void __launch_bounds__(kCountWarps * 32) k_count_box(TreeView tv, float3 lo, float3 hi,
+                                                                unsigned long long *cnt) {
+    __shared__ unsigned long long part[kCountWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // 0: outside, 1: cut, 2: inside
+    auto side = [&](int64_t node) {
+        const float4 a = __ldg(&tv.nlo[node]), b = __ldg(&tv.nhi[node]);
+        if (a.x > hi.x || b.x < lo.x || a.y > hi.y || b.y < lo.y || a.z > hi.z || b.z < lo.z) return 0;
+        return a.x >= lo.x && b.x <= hi.x && a.y >= lo.y && b.y <= hi.y && a.z >= lo.z && b.z <= hi.z ? 2 : 1;
+    };
+    const int64_t quarters = 4 * (tv.nlevels > 1 ? tv.cnt[1] : 1);
+    unsigned long long c = 0;  // this lane's points
+    for (int64_t w = (int64_t)blockIdx.x * kCountWarps + warp; w < quarters; w += (int64_t)gridDim.x * kCountWarps) {
+        const int64_t node = w >> 2, leaf0 = node * kFanout + 8 * (w & 3);
+        const int s1 = tv.nlevels > 1 ? side(tv.off[1] + node) : 1;  // warp-uniform
+        if (s1 == 0) continue;
+        const int64_t leaf = leaf0 + lane;
+        const int s0 = lane >= 8 || leaf >= tv.cnt[0] ? 0 : (s1 == 2 ? 2 : side(tv.off[0] + leaf));
+        if (s0 == 2) c += (unsigned long long)min((int64_t)kLeaf, tv.n - leaf * kLeaf);
+        for (unsigned m = __ballot_sync(0xffffffffu, s0 == 1); m;) {  // four leaves' loads at a time
+            float4 p[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                p[k] = make_float4(INFINITY, 0.f, 0.f, 0.f);  // outside
+                if (m) {
+                    const int64_t i = (leaf0 + __ffs(m) - 1) * kLeaf + lane;
+                    if (i < tv.n) p[k] = __ldg(&tv.pos[i]);
+                    m &= m - 1;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                c += p[k].x >= lo.x && p[k].x <= hi.x && p[k].y >= lo.y && p[k].y <= hi.y && p[k].z >= lo.z &&
+                     p[k].z <= hi.z;
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
+    if (lane == 0) part[warp] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kCountWarps; ++w) c += part[w];
+        if (c) atomicAdd(cnt, c);
+    }
+}
+
+cudaError_t launch_count_box(const sf_index *idx, float3 lo, float3 hi, unsigned long long *cnt, cudaStream_t s) {
+    const TreeView tv = idx->view();
+    const int64_t quarters = 4 * (tv.nlevels > 1 ? tv.cnt[1] : 1);
+    const unsigned g = std::max(1u, std::min<unsigned>(blocks_for(quarters, kCountWarps), 152 * 8));
+    return launch(k_count_box, dim3(g), dim3(kCountWarps * 32), 0, s, tv, lo, hi, cnt);
 }
 
 __global__ void k_set_params(DensityParams *dp, const unsigned long long *cnt, int64_t n_all,
@@ -79,9 +123,7 @@ sf_status set_density_params(sf_index *idx, bool clip, const sf_box &roi, const 
         lo = make_float3(flo[0], flo[1], flo[2]);
         hi = make_float3(fhi[0], fhi[1], fhi[2]);
         SF_TRY_CUDA(cudaMemsetAsync(cnt, 0, sizeof *cnt, s));
-        const unsigned g = std::max(1u, std::min<unsigned>(blocks_for(idx->n, 256), 152 * 8));
-        SF_TRY_CUDA(launch(k_count_box, dim3(g), dim3(256), 0, s, (const float4 *)idx->pos, idx->n,
-                           lo, hi, cnt));
+        SF_TRY_CUDA(launch_count_box(idx, lo, hi, cnt, s));
     }
     SF_TRY_CUDA(launch(k_set_params, dim3(1), dim3(1), 0, s, d_dp,
                        (const unsigned long long *)cnt, idx->n, ell[0], ell[1], ell[2], d_status));

@@ -322,9 +322,8 @@ struct GridSpec {
     double lo[3], hi[3], s[3];
 };
 
-// Count the points of a sorted cloud inside [lo, hi] (closed, float bounds) into *cnt.
-__global__ void k_count_box(const float4 *__restrict__ pos, int64_t n, float3 lo, float3 hi,
-                            unsigned long long *cnt);
+// Adds the number of the index's points inside [lo, hi] (closed, float bounds) to *cnt.
+cudaError_t launch_count_box(const sf_index *idx, float3 lo, float3 hi, unsigned long long *cnt, cudaStream_t s);
 // N_eff = *cnt (clip scope) or n_all (cnt == NULL), 1/N_eff and the uniform lengths
 // into *dp; ST_EMPTY into *status (nullable) when N_eff = 0.
 __global__ void k_set_params(DensityParams *dp, const unsigned long long *cnt, int64_t n_all,

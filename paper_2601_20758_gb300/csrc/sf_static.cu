@@ -169,10 +169,8 @@ extern "C" sf_status sf_kde_grid_static(sf_index *idx, const sf_box *roi, const 
         }
         // the count is left over from the previous call: clear it first
         SF_TRY_CUDA(cudaMemsetAsync(&S->count, 0, sizeof(unsigned long long), s));
-        const unsigned gb = std::max(1u, std::min<unsigned>(blocks_for(idx->n, 256), 152 * 8));
-        SF_TRY_CUDA(launch(k_count_box, dim3(gb), dim3(256), 0, s, (const float4 *)idx->pos, idx->n,
-                           make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]),
-                           &S->count));
+        SF_TRY_CUDA(launch_count_box(idx, make_float3(lo[0], lo[1], lo[2]), make_float3(hi[0], hi[1], hi[2]),
+                                     &S->count, s));
     }
     // so is the status word
     SF_TRY_CUDA(cudaMemsetAsync(&S->status, 0, sizeof(int), s));
