@@ -12,12 +12,14 @@
 // leaves (leaves whose support reaches the tile); the lists are cut into work
 // items of similar length; persistent warps drain the items, each lane owning
 // one (x, y) column of Z nodes in registers. Per candidate leaf the warp
-// refines its points (footprint in the tile, ROI clip), stages them in its own
-// shared memory with per-axis tables of the kernel factors at the tile's node
-// coordinates, so the inner loop per (point, node) pair is two instructions
-// (Gaussian: exp(a+b+c) = e^a e^b e^c with the truncation test on
-// q_x + q_y < 9 - q_z) or three (Epanechnikov). A last kernel adds each tile's
-// item partials in item order (deterministic). The allocation-free entry point
+// refines its points (footprint in the tile, ROI clip) and stages them in its
+// own shared memory; 32 at a time, across leaves, get per-axis tables of the
+// kernel factors at the tile's node coordinates, so the inner loop per (point,
+// node) pair is two instructions (Gaussian: exp(a+b+c) = e^a e^b e^c with the
+// truncation test on q_x + q_y < 9 - q_z) or three (Epanechnikov), and half of
+// one for the points whose support covers the whole tile. A tile of one item is
+// written by the work kernel; a last kernel adds the partials of the others in
+// item order (deterministic). The allocation-free entry point
 // keeps the older monolithic form: one CTA per 16 x 16 x 8 tile walking and
 // summing in one launch.
 //
@@ -837,20 +839,26 @@ __device__ __forceinline__ void mma_k8(float d[4], float a0, float a1, float a2,
 // Shared memory of one warp of the split pipeline: its 8 x 4 x TZ node tile. Rows of the
 // tables: the 32 staged particles being summed.
 constexpr int kWRing = 2 * kLeaf;  // staged particles: two halves of 32
-template <int TZ, bool ANISO>
+// x and y factors lie by groups of four particles, a node's four side by side, so that one
+// 16-byte load fetches them; the groups' padding keeps the fill's stores (one particle a
+// lane) off each other's banks.
+constexpr int kGX = 4 * kWX + 4, kGY = 4 * kWY + 4;
+template <int KER, int TZ, bool ANISO>
 struct __align__(16) WTileSmem {
-    float2 tx[kLeaf][kWX];   // Gauss: (c e^{-qx'}, qx'); Epan: (qx', -)
-    float2 ty[kLeaf][kWY];   // Gauss: (e^{-qy'}, qy');   Epan: (qy', -)
+    float xq[kLeaf / 4][kGX], yq[kLeaf / 4][kGY];  // q'
+    float xw[KER == SF_K_GAUSS3 ? kLeaf / 4 : 1][kGX];  // Gauss: c e^{-qx'}
+    float yw[KER == SF_K_GAUSS3 ? kLeaf / 4 : 1][kGY];  // Gauss: e^{-qy'}
     float tzw[kLeaf][TZ];    // Gauss: e^{-qz'};          Epan: c (1 - qz')
-    float tzl[kLeaf][TZ];    // Gauss: qmax - qz' (also the scratch of the tensor-core sums)
-    float cs[kLeaf];         // Epan: c
+    float tzl[KER == SF_K_GAUSS3 ? kLeaf : 1][TZ];  // Gauss: qmax - qz' (also the scratch of the tensor-core sums)
+    float cs[KER == SF_K_GAUSS3 ? 4 : kLeaf];       // Epan: c
     float4 sp[kWRing];       // staged (x, y, z, h)
     float4 sl[ANISO ? kWRing : 1];  // and (l_x, l_y, l_z)
     float2 axt[kWX + kWY + TZ];     // node coordinates (past the grid's end: the last node's again)
-    float uni[3];
-    EngineArgs e;
+    float uni[4];
     RoiDesc roi;
 };
+// four blocks of eight warps an SM
+static_assert(sizeof(WTileSmem<SF_K_GAUSS3, kTileZ, false>) <= (228 * 1024 / 4 - 1024) / 8, "tile tables");
 
 // Persistent warps: each takes (ROI, tile, leaf range) items from a counter and
 // sums them into the item's partial grid. No block barriers: a warp owns its
@@ -860,11 +868,14 @@ struct __align__(16) WTileSmem {
 // candidates are staged across leaves and summed 32 at a time (every lane fills one
 // particle's tables; one compensated fold per 32 particles, as for one full leaf), the
 // particles whose support covers the tile come first and are summed without a test, two
-// nodes an instruction (10 issue slots a particle and 256 nodes; 24 with the tests), and
-// table rows are written and read 16 bytes at a time. Work time (gaussian, kNN lengths) of a
-// 256^3 zoom of 67M points, 70% of whose staged particles cover their tile: 3.20 -> 1.88
-// ms; of its whole cube at 128^3 (supports of about a spacing): 3.74 -> 2.50 ms; 192^3 in
-// BF16: 1.34 -> 0.71 ms; 64 uneven grids: 48.8 -> 30.9 ms.
+// nodes an instruction (9 issue slots a particle and 256 nodes; 22 with the tests), and
+// shared memory, which took 83% of its cycles when every particle's x and y factors were
+// loaded by themselves, is read 16 bytes at a time (zoom below 1.92 -> 1.75 ms, 64 grids 30.8
+// -> 28.2; the group loops unrolled further: 1.78 and 29.3). Work time (gaussian, kNN lengths)
+// of a 256^3 zoom of 67M points, 70% of whose staged particles cover their tile, against one
+// leaf staged at a time and every pair tested: 3.20 -> 1.75 ms; of its whole cube at 128^3
+// (supports of about a spacing): 3.74 -> 2.56 ms; 192^3 in BF16: 1.34 -> 0.73 ms; 64 uneven
+// grids: 48.8 -> 28.2 ms.
 template <int KER, int BW, bool CLIP, bool CNT, int TZ, int PREC = SF_PREC_FP32>
 __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
     k_mr_work(MrArgs a, const int4 *__restrict__ items, const uint32_t *__restrict__ n_items,
@@ -874,7 +885,7 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
     constexpr bool kMma = KER == SF_K_GAUSS3 && TZ == 8 && PREC != SF_PREC_FP32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    typedef WTileSmem<TZ, BW == BW_ANISO> Smem;
+    typedef WTileSmem<KER, TZ, BW == BW_ANISO> Smem;
     Smem &S = reinterpret_cast<Smem *>(smem_raw)[warp];
     const int cx = lane & (kWX - 1), cy = lane / kWX;
     const unsigned lt = (1u << lane) - 1u;
@@ -889,14 +900,11 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
         const int4 it = items[item];
         const int ri = a.tile_roi ? a.tile_roi[it.x] : 0;
         if (ri != cur_roi) {
-            if (lane == 0) {
-                S.roi = a.rois[ri];
-                set_roi_engine(S.e, a.e, S.roi);
-            }
+            if (lane == 0) S.roi = a.rois[ri];
             cur_roi = ri;
             __syncwarp();
         }
-        const EngineArgs &E = S.e;
+        const EngineArgs &E = a.e;
         const RoiDesc &r = S.roi;
         // ---- the tile's node coordinates
         int gx0, gy0, gz0, nv[3];
@@ -909,9 +917,9 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
             S.axt[lane] = v;
         }
         if (lane == 0) {
-            S.uni[0] = E.dp->ell_uniform[0];
-            S.uni[1] = E.dp->ell_uniform[1];
-            S.uni[2] = E.dp->ell_uniform[2];
+            S.uni[0] = r.dp->ell_uniform[0];
+            S.uni[1] = r.dp->ell_uniform[1];
+            S.uni[2] = r.dp->ell_uniform[2];
         }
         __syncwarp();
         float mcen[3], mhw[3];  // the tile box widened by the rounding margin, as centre and half-width
@@ -955,8 +963,8 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                     point_ell<BW>(E, S.uni, i, p, l);
                     ok = l[0] > 0.f && l[1] > 0.f && l[2] > 0.f;
                     if (CLIP)
-                        ok = ok && p.x >= E.blo[0] && p.x <= E.bhi[0] && p.y >= E.blo[1] &&
-                             p.y <= E.bhi[1] && p.z >= E.blo[2] && p.z <= E.bhi[2];
+                        ok = ok && p.x >= r.blo[0] && p.x <= r.bhi[0] && p.y >= r.blo[1] &&
+                             p.y <= r.bhi[1] && p.z >= r.blo[2] && p.z <= r.bhi[2];
                     const float pc[3] = {p.x, p.y, p.z};
                     float rl[3], qlb = 0.f;
                     bool small = false;
@@ -1019,8 +1027,9 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
             const int ns = min(staged, kLeaf);
             __syncwarp();
             bool full = false;  // the support covers every node of the tile
-            float mx = 0.f, my = 0.f, mz = 0.f, c = 0.f, u[3] = {0.f, 0.f, 0.f};
-            float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+            // lanes past the last particle: one infinitely far, which adds nothing
+            float c = 1.f, u[3] = {1.f, 1.f, 1.f};
+            float4 p = make_float4(INFINITY, 0.f, 0.f, 0.f);
             if (lane < ns) {
                 const int e = head + lane;
                 p = S.sp[e];
@@ -1045,9 +1054,9 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                     const float t0 = ((n0.x - pc) + n0.y) * uu, t1 = ((n1.x - pc) + n1.y) * uu;
                     return fmaxf(t0 * t0, t1 * t1);
                 };
-                mx = ends(0, kWX, p.x, u[0]);
-                my = ends(kWX, kWY, p.y, u[1]);
-                mz = ends(kWX + kWY, TZ, p.z, u[2]);
+                const float mx = ends(0, kWX, p.x, u[0]);
+                const float my = ends(kWX, kWY, p.y, u[1]);
+                const float mz = ends(kWX + kWY, TZ, p.z, u[2]);
                 if (KER == SF_K_GAUSS3) full = mx + my < KDef<KER>::qmax - mz;
                 else full = c * (1.0f - mz) - c * (mx + my) > 0.f;
             }
@@ -1055,32 +1064,33 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
             const unsigned balf = __ballot_sync(0xffffffffu, full);
             const int nf = __popc(balf);
             if (CNT && lane == 0 && KER == SF_K_GAUSS3 && TZ == 8) st_full += nf;
-            if (lane < ns) {
+            // some row is tested (warp-uniform): rows are taken by fours
+            const bool tests = CNT || KER != SF_K_GAUSS3 || nf < ns || (ns & 3) != 0;
+            {
                 const int s = full ? __popc(balf & lt) : nf + __popc(~balf & lt);
                 auto q_at = [&](float2 nc, float pc, float uu) {
                     const float t = ((nc.x - pc) + nc.y) * uu;
                     return t * t;
                 };
-                // two nodes of x or y a step, four of z, in an order that starts by the row so
-                // that the lanes' 16-byte stores spread over the banks
+                const int g = s >> 2, sl = s & 3;
+                auto axis = [&](auto put, int off, int n, float pc, float uu) {  // nodes two at a time
 #pragma unroll
-                for (int t = 0; t < kWX / 2; ++t) {
-                    const int i = 2 * ((t + (s >> 1)) & (kWX / 2 - 1));
-                    const float4 nc = *reinterpret_cast<const float4 *>(&S.axt[i]);
-                    const float q0 = q_at(make_float2(nc.x, nc.y), p.x, u[0]), q1 = q_at(make_float2(nc.z, nc.w), p.x, u[0]);
-                    *reinterpret_cast<float4 *>(&S.tx[s][i]) =
-                        KER == SF_K_GAUSS3 ? make_float4(ex2_approx(-q0) * c, q0, ex2_approx(-q1) * c, q1)
-                                           : make_float4(q0, 0.f, q1, 0.f);
-                }
-#pragma unroll
-                for (int t = 0; t < kWY / 2; ++t) {
-                    const int i = 2 * ((t + (s >> 2)) & (kWY / 2 - 1));
-                    const float4 nc = *reinterpret_cast<const float4 *>(&S.axt[kWX + i]);
-                    const float q0 = q_at(make_float2(nc.x, nc.y), p.y, u[1]), q1 = q_at(make_float2(nc.z, nc.w), p.y, u[1]);
-                    *reinterpret_cast<float4 *>(&S.ty[s][i]) =
-                        KER == SF_K_GAUSS3 ? make_float4(ex2_approx(-q0), q0, ex2_approx(-q1), q1)
-                                           : make_float4(q0, 0.f, q1, 0.f);
-                }
+                    for (int i = 0; i < n; i += 2) {
+                        const float4 nc = *reinterpret_cast<const float4 *>(&S.axt[off + i]);
+                        put(i, q_at(make_float2(nc.x, nc.y), pc, uu));
+                        put(i + 1, q_at(make_float2(nc.z, nc.w), pc, uu));
+                    }
+                };
+                axis([&](int i, float q) {
+                    if (KER == SF_K_GAUSS3) S.xw[g][4 * i + sl] = ex2_approx(-q) * c;
+                    if (tests) S.xq[g][4 * i + sl] = q;
+                }, 0, kWX, p.x, u[0]);
+                axis([&](int i, float q) {
+                    if (KER == SF_K_GAUSS3) S.yw[g][4 * i + sl] = ex2_approx(-q);
+                    if (tests) S.yq[g][4 * i + sl] = q;
+                }, kWX, kWY, p.y, u[1]);
+                // four nodes of z a step, in an order that starts by the row so that the lanes'
+                // 16-byte stores spread over the banks
 #pragma unroll
                 for (int t = 0; t < TZ / 4; ++t) {
                     const int i = 4 * ((t + (s >> 2)) & (TZ / 4 - 1));
@@ -1092,7 +1102,8 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                         *reinterpret_cast<float4 *>(&S.tzw[s][i]) =
                             make_float4(ex2_approx(-q0), ex2_approx(-q1), ex2_approx(-q2), ex2_approx(-q3));
                         constexpr float qm = KDef<KER>::qmax;
-                        *reinterpret_cast<float4 *>(&S.tzl[s][i]) = make_float4(qm - q0, qm - q1, qm - q2, qm - q3);
+                        if (tests)
+                            *reinterpret_cast<float4 *>(&S.tzl[s][i]) = make_float4(qm - q0, qm - q1, qm - q2, qm - q3);
                     } else {
                         *reinterpret_cast<float4 *>(&S.tzw[s][i]) =
                             make_float4(c * (1.0f - q0), c * (1.0f - q1), c * (1.0f - q2), c * (1.0f - q3));
@@ -1103,63 +1114,80 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
             __syncwarp();
             head ^= kLeaf;
             staged -= ns;
-            // ---- accumulate: lane owns column (cx, cy) and TZ nodes in z
-            const int s_test = CNT ? 0 : nf;  // rows from here on are tested
-            if (!kMma && !CNT) {
+            // ---- accumulate: lane owns column (cx, cy) and TZ nodes in z; four rows at a time
+            auto four = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
+            const int gf = CNT || kMma ? 0 : nf >> 2;  // groups of full rows
+            if (gf > 0) {
                 f32x2 acc2[TZ / 2];
 #pragma unroll
                 for (int k = 0; k < TZ / 2; ++k) acc2[k] = f2_pack(acc[2 * k], acc[2 * k + 1]);
-#pragma unroll 4
-                for (int s = 0; s < nf; ++s) {
-                    float b;
-                    if (KER == SF_K_GAUSS3) b = S.tx[s][cx].x * S.ty[s][cy].x;
-                    else b = S.cs[s] * (S.tx[s][cx].x + S.ty[s][cy].x);
-                    const f32x2 bb = f2_pack(b, b);
+#pragma unroll 1
+                for (int g = 0; g < gf; ++g) {
+                    float bv[4];
+                    if (KER == SF_K_GAUSS3) {
+                        const float4 X = four(&S.xw[g][4 * cx]), Y = four(&S.yw[g][4 * cy]);
+                        bv[0] = X.x * Y.x; bv[1] = X.y * Y.y; bv[2] = X.z * Y.z; bv[3] = X.w * Y.w;
+                    } else {
+                        const float4 X = four(&S.xq[g][4 * cx]), Y = four(&S.yq[g][4 * cy]), C = four(&S.cs[4 * g]);
+                        bv[0] = C.x * (X.x + Y.x); bv[1] = C.y * (X.y + Y.y);
+                        bv[2] = C.z * (X.z + Y.z); bv[3] = C.w * (X.w + Y.w);
+                    }
 #pragma unroll
-                    for (int k = 0; k < TZ; k += 4) {
-                        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(&S.tzw[s][k]);
-                        if (KER == SF_K_GAUSS3) {
-                            acc2[k / 2] = f2_fma(bb, z.x, acc2[k / 2]);
-                            acc2[k / 2 + 1] = f2_fma(bb, z.y, acc2[k / 2 + 1]);
-                        } else {
-                            acc2[k / 2] = f2_add(acc2[k / 2], f2_sub(z.x, bb));
-                            acc2[k / 2 + 1] = f2_add(acc2[k / 2 + 1], f2_sub(z.y, bb));
+                    for (int j = 0; j < 4; ++j) {
+                        const f32x2 bb = f2_pack(bv[j], bv[j]);
+#pragma unroll
+                        for (int k = 0; k < TZ; k += 4) {
+                            const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(&S.tzw[4 * g + j][k]);
+                            if (KER == SF_K_GAUSS3) {
+                                acc2[k / 2] = f2_fma(bb, z.x, acc2[k / 2]);
+                                acc2[k / 2 + 1] = f2_fma(bb, z.y, acc2[k / 2 + 1]);
+                            } else {
+                                acc2[k / 2] = f2_add(acc2[k / 2], f2_sub(z.x, bb));
+                                acc2[k / 2 + 1] = f2_add(acc2[k / 2 + 1], f2_sub(z.y, bb));
+                            }
                         }
                     }
                 }
 #pragma unroll
                 for (int k = 0; k < TZ / 2; ++k) f2_unpack(acc2[k], acc[2 * k], acc[2 * k + 1]);
             }
-#pragma unroll 2
-            for (int s = kMma ? nf : s_test; s < ns; ++s) {
-                const float2 ex = S.tx[s][cx];
-                const float2 ey = S.ty[s][cy];
+            // the groups from the first with a row that is not full (rows past the last particle
+            // add nothing); with the tensor cores the full rows are theirs
+#pragma unroll 1
+            for (int g = kMma ? nf >> 2 : gf; 4 * g < ns; ++g) {
+                const float4 X = four(&S.xq[g][4 * cx]), Y = four(&S.yq[g][4 * cy]);
+                const float qv[4] = {X.x + Y.x, X.y + Y.y, X.z + Y.z, X.w + Y.w};
+                float bv[4];
                 if (KER == SF_K_GAUSS3) {
-                    const float bse = ex.x * ey.x;
-                    const float qij = ex.y + ey.y;
-#pragma unroll
-                    for (int k = 0; k < TZ; k += 4) {
-                        const float4 w = *reinterpret_cast<const float4 *>(&S.tzw[s][k]);
-                        const float4 m = *reinterpret_cast<const float4 *>(&S.tzl[s][k]);
-                        const float wv[4] = {w.x, w.y, w.z, w.w}, mv[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (qij < mv[j]) {
-                                acc[k + j] = fmaf(bse, wv[j], acc[k + j]);
-                                if (CNT && k + j < nv[2]) ++np;
-                            }
-                    }
+                    const float4 V = four(&S.xw[g][4 * cx]), W = four(&S.yw[g][4 * cy]);
+                    bv[0] = V.x * W.x; bv[1] = V.y * W.y; bv[2] = V.z * W.z; bv[3] = V.w * W.w;
                 } else {
-                    const float b = S.cs[s] * (ex.x + ey.x);
+                    const float4 C = four(&S.cs[4 * g]);
+                    bv[0] = C.x * qv[0]; bv[1] = C.y * qv[1]; bv[2] = C.z * qv[2]; bv[3] = C.w * qv[3];
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (kMma && 4 * g + j < nf) continue;
 #pragma unroll
                     for (int k = 0; k < TZ; k += 4) {
-                        const float4 w = *reinterpret_cast<const float4 *>(&S.tzw[s][k]);
+                        const float4 w = four(&S.tzw[4 * g + j][k]);
                         const float wv[4] = {w.x, w.y, w.z, w.w};
+                        if (KER == SF_K_GAUSS3) {
+                            const float4 m = four(&S.tzl[4 * g + j][k]);
+                            const float mv[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float t = wv[j] - b;
-                            acc[k + j] += fmaxf(t, 0.f);
-                            if (CNT && k + j < nv[2]) np += (t > 0.f);
+                            for (int i = 0; i < 4; ++i)
+                                if (qv[j] < mv[i]) {
+                                    acc[k + i] = fmaf(bv[j], wv[i], acc[k + i]);
+                                    if (CNT && k + i < nv[2]) ++np;
+                                }
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float t = wv[i] - bv[j];
+                                acc[k + i] += fmaxf(t, 0.f);
+                                if (CNT && k + i < nv[2]) np += (t > 0.f);
+                            }
                         }
                     }
                 }
@@ -1174,10 +1202,10 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                         for (int e = 0; e < 4; ++e) {
                             const int sp = s0 + 2 * tig + (e & 1) + 8 * (e >> 1);
                             const bool v = sp < nf;
-                            ax[e] = v ? S.tx[sp][gq].x : 0.f;
+                            ax[e] = v ? S.xw[sp >> 2][4 * gq + (sp & 3)] : 0.f;
                             bz[e] = v ? S.tzw[sp][gq] : 0.f;
 #pragma unroll
-                            for (int y = 0; y < 4; ++y) ay[e][y] = v ? S.ty[sp][y].x : 0.f;
+                            for (int y = 0; y < 4; ++y) ay[e][y] = v ? S.yw[sp >> 2][4 * y + (sp & 3)] : 0.f;
                         }
                         const uint32_t b0 = bf16x2_of(bz[0], bz[1]), b1 = bf16x2_of(bz[2], bz[3]);
 #pragma unroll
@@ -1194,12 +1222,12 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                     for (int s0 = 0; s0 < nf; s0 += 8) {
                         const int sa = s0 + tig, sb = s0 + tig + 4;
                         const bool va = sa < nf, vb = sb < nf;
-                        const float txa = va ? S.tx[sa][gq].x : 0.f, txb = vb ? S.tx[sb][gq].x : 0.f;
+                        const float txa = va ? S.xw[sa >> 2][4 * gq + (sa & 3)] : 0.f, txb = vb ? S.xw[sb >> 2][4 * gq + (sb & 3)] : 0.f;
                         const float tza = va ? S.tzw[sa][gq] : 0.f, tzb = vb ? S.tzw[sb][gq] : 0.f;
 #pragma unroll
                         for (int mb = 0; mb < 2; ++mb) {
-                            const float ya0 = va ? S.ty[sa][2 * mb].x : 0.f, ya1 = va ? S.ty[sa][2 * mb + 1].x : 0.f;
-                            const float yb0 = vb ? S.ty[sb][2 * mb].x : 0.f, yb1 = vb ? S.ty[sb][2 * mb + 1].x : 0.f;
+                            const float ya0 = va ? S.yw[sa >> 2][8 * mb + (sa & 3)] : 0.f, ya1 = va ? S.yw[sa >> 2][8 * mb + 4 + (sa & 3)] : 0.f;
+                            const float yb0 = vb ? S.yw[sb >> 2][8 * mb + (sb & 3)] : 0.f, yb1 = vb ? S.yw[sb >> 2][8 * mb + 4 + (sb & 3)] : 0.f;
                             mma_k8<PREC>(mb ? d1 : d0, txa * ya0, txa * ya1, txb * yb0, txb * yb1, tza, tzb);
                         }
                     }
@@ -1409,14 +1437,14 @@ static sf_status mr_count(const MrArgs &a, uint32_t *cnt, uint32_t *off, uint32_
     return SF_OK;
 }
 
-template <int TZ, int BW>
+template <int KER, int TZ, int BW>
 static size_t mr_work_smem() {
-    return sizeof(WTileSmem<TZ, BW == BW_ANISO>) * (kGridThreads / 32);
+    return sizeof(WTileSmem<KER, TZ, BW == BW_ANISO>) * (kGridThreads / 32);
 }
 
 template <int KER, int BW, bool CLIP, bool CNT, int TZ>
 static sf_status mr_work_attr(int *per_sm) {
-    const size_t smem = mr_work_smem<TZ, BW>();
+    const size_t smem = mr_work_smem<KER, TZ, BW>();
     static std::atomic<uint64_t> attr{0};
     SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ>, smem, attr));
     SF_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_mr_work<KER, BW, CLIP, CNT, TZ>,
@@ -1439,9 +1467,9 @@ struct MrBuffers {
 template <int KER, int BW, bool CLIP, bool CNT, int TZ, int PREC>
 static sf_status launch_work(const MrArgs &a, const MrBuffers &b, cudaStream_t s) {
     static std::atomic<uint64_t> attr{0};
-    SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, mr_work_smem<TZ, BW>(), attr));
+    SF_TRY_CUDA(smem_attr_once(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, mr_work_smem<KER, TZ, BW>(), attr));
     SF_TRY_CUDA(launch(k_mr_work<KER, BW, CLIP, CNT, TZ, PREC>, dim3((unsigned)b.slots), dim3(kGridThreads),
-                       mr_work_smem<TZ, BW>(), s, a, (const int4 *)b.items, (const uint32_t *)(b.tot + 1),
+                       mr_work_smem<KER, TZ, BW>(), s, a, (const int4 *)b.items, (const uint32_t *)(b.tot + 1),
                        (const int *)b.list, b.part, b.next));
     return SF_OK;
 }
