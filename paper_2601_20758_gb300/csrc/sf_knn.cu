@@ -1298,8 +1298,8 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
     a.next_leaf = counters;
     KTimer timer(d_work ? "k_knn_count" : "k_knn", s);
     if (!d_nbr_orig) {  // the neighbour ids are k_knn's
-        // Lists of CAP entries: between leaves CAP - 32 of them, which have to hold k and
-        // kSelExtra and leave room, so that few leaves force a compaction; shared
+        // Lists of CAP entries: between leaves CAP - 32 of them, which have to hold k and the
+        // boundary's ties and leave room, so that few leaves force a compaction; shared
         // memory (128 bytes a row and warp) sets how many warps an SM holds.
         KnnSelArgs b;
         b.tv = a.tv;
