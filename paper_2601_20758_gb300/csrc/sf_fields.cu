@@ -114,10 +114,11 @@ __global__ void __launch_bounds__(kRsX * kRsY)
         const int64_t row = A.n[0], slice = (int64_t)A.n[0] * A.n[1];
         float *d = dst + ((int64_t)g0[2] * A.dn[1] + iy) * A.dn[0] + ix;
         const int64_t dslice = (int64_t)A.dn[0] * A.dn[1];
+        const float zero = weight * 0.f;  // a negative weight's zero is -0
 #pragma unroll 2
         for (int z = 0; z < nz; ++z) {
             const AxisPlace pz = P[kRsX + kRsY + z];
-            float res = 0.f;
+            float res = zero;
             if (px.c >= 0 && py.c >= 0 && pz.c >= 0) {
                 const float *f = src + pz.c * slice + py.c * row + px.c;
                 const float f000 = __ldg(f), f100 = __ldg(f + 1);
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kRsX * kRsY)
                 // are exact
                 const bool plain = (int)any >= 0 && fabsf(hi) > 1.0e-28f && fabsf(hi) < 1.0e37f &&
                                    ((fabsf(r) > 1.0e-28f && fabsf(r) < 1.0e37f) || weight == 0.f);
-                if (!plain) res = any ? resample_fp64(src, A, weight, ix, iy, g0[2] + z) : 0.f;
+                if (!plain) res = any ? resample_fp64(src, A, weight, ix, iy, g0[2] + z) : zero;
             } else {
                 ++out_cnt;
             }

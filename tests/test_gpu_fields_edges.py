@@ -74,6 +74,15 @@ def test_resample_edges(field, dims, dst, weight):
         assert np.array_equal(got[inf & ~near_max], ref32[inf & ~near_max])
 
 
+def test_resample_negative_weight_gives_negative_zero():
+    # zero times a negative weight is -0, inside the box and outside
+    out = torch.full((4 * 4 * 4,), 7.0, device="cuda")
+    n_out = L.sf_resample_grid(torch.zeros(27, device="cuda"), L.make_box((0, 0, 0), (1, 1, 1)), (3, 3, 3),
+                               L.make_box((0, 0, 0), (1.5, 1, 1)), (4, 4, 4), out, weight=-2.0, want_outside=True)
+    got = out.cpu().numpy()
+    assert n_out == 16 and not got.any() and np.signbit(got).all()
+
+
 @pytest.mark.parametrize("dims", [(2, 2, 2), (3, 2, 40), (33, 2, 2), (17, 33, 9), (130, 5, 4), (64, 64, 3)])
 @pytest.mark.parametrize("t", [0.5, 0.97, 0.0, -1e300, 1e300, float(np.float32(0.25)), 0.25 + 2.0 ** -40])
 def test_iso_edges(dims, t):
