@@ -1072,7 +1072,11 @@ struct KnnSel {
                 cum += (int)S.list[b][lane];
                 if (cum > a.k) break;  // the point itself is counted
             }
-            T = b < 31 && base + b >= 0 ? fminf(__uint_as_float(((uint32_t)(base + b + 1) << 21) - 1u), far) : far;
+            // The margin (as k_knn's) is the rounding of FP32 d2: the point FP32 puts just above the
+            // bin's edge may be nearer than the one it puts just below.
+            T = b < 31 && base + b >= 0
+                    ? fminf(__uint_as_float((uint32_t)(base + b + 1) << 21) * (1.0f + 4.0e-6f), far)
+                    : far;
             if (!valid) T = -1.f;
             __syncwarp();
         }
