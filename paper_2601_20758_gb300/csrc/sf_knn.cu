@@ -51,14 +51,14 @@ struct KnnWarpSmem {
     float4 blo[32], bhi[32];   // child boxes under test
     float4 pts[kLeaf];         // staged candidates (x, y, z, original id bits)
     uint32_t hist[kNB][32];
+    unsigned left;             // lanes left to a finer scale
 };
 
 struct KnnArgs {
     TreeView tv;
     const uint32_t *perm;
     int k;
-    float scale;              // power of two applied to every coordinate
-    double unscale2;          // 1 / scale^2
+    float scale;              // power of two applied to every coordinate (first try)
     float *h_sorted;          // out: h per sorted point
     uint32_t *nbr_orig;       // out (nullable): [n][k] by original index
     int *leaf_list;           // [slots][kLeafList] accepted leaves of the current query leaf
@@ -71,8 +71,11 @@ struct KnnArgs {
     const unsigned int *retry_n;
 };
 
-// Coordinates are scaled by a power of two on load (exact) so that the cloud's extent is
-// about 2^30: FP32 d2 then neither overflows nor, down to 2^-90 of the extent, underflows.
+// Coordinates are scaled by a power of two on load, first to an extent of about 2^30, then
+// for the lanes whose k-th point lies within 2^-30 of their bracket's radius (a point far
+// out widens it), or whose bracket is below 1, to 2^30 times that, and so on: the k-th
+// FP32 d2 neither overflows nor underflows. Scaling up is exact; scaling down loses bits below
+// 2^-149, which FP64 distances of 2^-30 and more do not see.
 __device__ __forceinline__ float4 ld_scaled(const float4 *p, float scale) {
     float4 v = __ldg(p);
     v.x *= scale;
@@ -330,16 +333,20 @@ struct KnnWarp {
     }
 };
 
-template <bool COUNT>
-__device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint32_t *leaf_mask, double *bd, uint32_t *bi,
-                         int64_t leaf) {
+// The leaf's queries at the first scale, or (FINER) those of `lanes` at finer_scale; S.left gets
+// the lanes left to a finer one.
+template <bool COUNT, bool FINER>
+__device__ __forceinline__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint32_t *leaf_mask,
+                                         double *bd, uint32_t *bi, int64_t leaf, float finer_scale = 0.f,
+                                         unsigned lanes = 0xffffffffu) {
+    const float scale = FINER ? finer_scale : a.scale;
     const int lane = threadIdx.x & 31;
     const TreeView &tv = a.tv;
     const int k = a.k;
     const int64_t qi = leaf * kLeaf + lane;
-    const bool valid = qi < tv.n;
-    KnnWarp<COUNT> W(tv, a.perm, a.scale, S, leaf_list, leaf_mask);
-    W.q = valid ? ld_scaled(&tv.pos[qi], a.scale) : make_float4(0.f, 0.f, 0.f, 0.f);
+    bool valid = qi < tv.n && (!FINER || ((lanes >> lane) & 1u));
+    KnnWarp<COUNT> W(tv, a.perm, scale, S, leaf_list, leaf_mask);
+    W.q = valid ? ld_scaled(&tv.pos[qi], scale) : make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 q = W.q;
     const uint32_t qid = valid ? __ldg(&a.perm[qi]) : 0u;
 
@@ -370,18 +377,19 @@ __device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint3
     {
         float blo[3] = {INFINITY, INFINITY, INFINITY}, bhi[3] = {-INFINITY, -INFINITY, -INFINITY};
         for (int64_t L = c0; L <= c1; ++L) {
-            const float4 lo = ld_scaled(&tv.nlo[L], a.scale), hi = ld_scaled(&tv.nhi[L], a.scale);
+            const float4 lo = ld_scaled(&tv.nlo[L], scale), hi = ld_scaled(&tv.nhi[L], scale);
             blo[0] = fminf(blo[0], lo.x); blo[1] = fminf(blo[1], lo.y); blo[2] = fminf(blo[2], lo.z);
             bhi[0] = fmaxf(bhi[0], hi.x); bhi[1] = fmaxf(bhi[1], hi.y); bhi[2] = fmaxf(bhi[2], hi.z);
         }
         const float dx = fmaxf(q.x - blo[0], bhi[0] - q.x), dy = fmaxf(q.y - blo[1], bhi[1] - q.y),
                     dz = fmaxf(q.z - blo[2], bhi[2] - q.z);
         whi = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * (1.0f + 1.0e-5f);
+        if (FINER) whi = fminf(whi, 0x1p64f);  // no bracket was wider in the coarser scale
     }
     auto window_visit = [&](int64_t L0, int64_t L1, auto fn) {
         for (int64_t L = L0; L <= L1; ++L) {
             const int64_t base = L * kLeaf;
-            if (base + lane < tv.n) S.pts[lane] = ld_scaled(&tv.pos[base + lane], a.scale);
+            if (base + lane < tv.n) S.pts[lane] = ld_scaled(&tv.pos[base + lane], scale);
             __syncwarp();
             const int cnt = (int)(tv.n - base < kLeaf ? tv.n - base : kLeaf);
             for (int t = 0; t < cnt; ++t) fn(S.pts[t], base + t);
@@ -415,6 +423,24 @@ __device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint3
             const float nhi = (b == kNB - 1 ? whi : wlo + (float)(b + 1) * (width / (float)kNB)) *
                               (1.0f + 1.0e-6f);
             whi = fminf(nhi, whi);
+        }
+        if (round == 1) {  // a finer scale?
+            const bool room = valid && scale < 0x1p96f && fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fabsf(q.z)) < 0x1p96f;
+            unsigned left = 0;
+            if (__any_sync(0xffffffffu, room && (b == 0 || whi < 1.0f))) {
+                int near = 0, same = 0;
+                const float lim = whi < 1.0f ? whi : whi * 0x1p-60f;
+                window_visit(w0, w1, [&](float4 p, int64_t j) {
+                    if (j != qi && d2_f32(q, p) <= lim) {
+                        ++near;
+                        same += p.x == q.x && p.y == q.y && p.z == q.z;  // at distance 0 in any scale
+                    }
+                });
+                left = __ballot_sync(0xffffffffu, room && near >= k && same < k);
+                valid = valid && !((left >> lane) & 1u);
+            }
+            if (lane == 0) S.left = left;
+            if (!__any_sync(0xffffffffu, valid)) return;
         }
     }
     const float T = valid ? whi * (1.0f + 4.0e-6f) + 1.0e-37f : -1.f;
@@ -545,8 +571,8 @@ __device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint3
                 const int pick = min(max(need, 1), min(nband, kBand)) - 1;
                 kth = bd[pick * 32 + lane];
                 done = true;
-            } else if (round == 7 || !(e_hi - e_lo > 4.0f * kDelta * e_hi)) {
-                extract = true;  // bin cannot shrink further (or out of rounds)
+            } else if (round == 7 || !(e_hi - e_lo > fmaxf(4.0f * kDelta * e_hi, 1.0e-37f))) {
+                extract = true;  // bin cannot shrink further (kNB / width would overflow), or out of rounds
             } else {
                 lo_e = e_lo;     // the band pass already binned [e_lo, e_hi]
                 hi_e = e_hi;
@@ -592,7 +618,10 @@ __device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint3
             }
         }
     }
-    if (valid) a.h_sorted[qi] = (float)sqrt(kth * a.unscale2);
+    if (valid) {
+        const double inv = 1.0 / (double)scale;  // a power of two
+        a.h_sorted[qi] = (float)sqrt(kth * (inv * inv));
+    }
 
     // ---- optional neighbour ids: the below set, then the band's first `need`
     if (a.nbr_orig) {
@@ -609,12 +638,18 @@ __device__ void knn_leaf(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint3
     }
     if (COUNT && lane == 0) {
         atomicAdd(&a.work[0], W.ncand);
-        atomicAdd(&a.work[1], 1ull);
+        if (S.left == 0) atomicAdd(&a.work[1], 1ull);
     }
 }
 
 template <bool COUNT>
-__global__ void __launch_bounds__(kKnnWarps * 32, 7) k_knn(KnnArgs a) {
+__device__ __noinline__ void knn_leaf_finer(const KnnArgs &a, KnnWarpSmem &S, int *leaf_list, uint32_t *leaf_mask,
+                                            double *bd, uint32_t *bi, int64_t leaf, float scale, unsigned lanes) {
+    knn_leaf<COUNT, true>(a, S, leaf_list, leaf_mask, bd, bi, leaf, scale, lanes);
+}
+
+template <bool COUNT>
+__global__ void __launch_bounds__(kKnnWarps * 32, 7) k_knn(const __grid_constant__ KnnArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5;
     KnnWarpSmem &S = reinterpret_cast<KnnWarpSmem *>(smem_raw)[warp];
@@ -630,7 +665,15 @@ __global__ void __launch_bounds__(kKnnWarps * 32, 7) k_knn(KnnArgs a) {
         leaf = __shfl_sync(0xffffffffu, leaf, 0);
         if ((int64_t)leaf >= nleaf) break;
         if (a.retry) leaf = a.retry[leaf];
-        knn_leaf<COUNT>(a, S, leaf_list, leaf_mask, bd, bi, (int64_t)leaf);
+        knn_leaf<COUNT, false>(a, S, leaf_list, leaf_mask, bd, bi, (int64_t)leaf);
+        __syncwarp();
+        float scale = a.scale;
+        while (const unsigned left = S.left) {  // ends: none is left past 2^96
+            __syncwarp();
+            scale *= 0x1p30f;
+            knn_leaf_finer<COUNT>(a, S, leaf_list, leaf_mask, bd, bi, (int64_t)leaf, scale, left);
+            __syncwarp();
+        }
     }
 }
 
@@ -1290,11 +1333,15 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
     a.nbr_orig = d_nbr_orig;
     a.work = d_work;
     a.retry = a.retry_n = nullptr;
-    float extent = 0.f;
-    for (int d = 0; d < 3; ++d) extent = std::max(extent, idx->bbox_hi[d] - idx->bbox_lo[d]);
-    const int e = std::isfinite(extent) && extent > 0.f ? std::min(std::max(30 - std::ilogb(extent), -126), 127) : 0;
-    a.scale = std::ldexp(1.0f, e);
-    a.unscale2 = std::ldexp(1.0, -2 * e);
+    float extent = 0.f, most = 0.f;
+    for (int d = 0; d < 3; ++d) {
+        extent = std::max(extent, idx->bbox_hi[d] - idx->bbox_lo[d]);
+        most = std::max(most, std::max(std::fabs(idx->bbox_lo[d]), std::fabs(idx->bbox_hi[d])));
+    }
+    // differences of at most 2^31, and the largest coordinate stays finite
+    const int e = std::min(30 - (std::isfinite(extent) ? (extent > 0.f ? std::ilogb(extent) : 30) : 128),
+                           most > 0.f ? 126 - std::ilogb(most) : 0);
+    a.scale = std::ldexp(1.0f, std::min(e, 126));
     Scratch sc(s);
     unsigned int *counters = sc.get<unsigned int>(5);  // next leaf of three kernels, two retry counts
     SF_TRY_SCRATCH(sc);

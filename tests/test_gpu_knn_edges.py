@@ -1,7 +1,8 @@
 """kNN bandwidths bit for bit where FP32 and FP64 order two points differently across a
 power-of-two fraction (the edges of the search's distance bins): the k-th nearest point is
 the one whose FP32 squared distance lies on the edge, a farther one's just below it. Alone
-(the first bound decides) and with a shell of points that makes the lists overflow."""
+(the first bound decides) and with a shell of points that makes the lists overflow. And
+where FP32 squares leave its range, next to distances or coordinates of another scale."""
 import numpy as np
 import pytest
 import torch
@@ -37,6 +38,26 @@ def _swapped(q, edge, r):
     return a, b
 
 
+def _check(xyz, k):
+    xyz = np.ascontiguousarray(xyz, dtype=F)
+    idx = L.sf_build_index(torch.from_numpy(xyz).cuda())
+    try:
+        L.sf_bandwidths(idx, L.make_params(k=k))
+        h = torch.empty(len(xyz), device="cuda")
+        L.sf_get_bandwidths(idx, h)
+        nbr = torch.empty((len(xyz), k), dtype=torch.int32, device="cuda")
+        h2 = torch.empty_like(h)
+        L.sf_knn_neighbours(idx, k, nbr, h2)
+        torch.cuda.synchronize()
+    finally:
+        L.sf_free_index(idx)
+    ref = np.asarray(oracle.knn(xyz, k)[0], dtype=F)
+    assert np.array_equal(h.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+    assert np.array_equal(h2.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+    far = np.stack([np.sort(_d2_f64(xyz[i], xyz[nbr[i].cpu().numpy()]))[-1] for i in range(0, len(xyz), 97)])
+    assert np.array_equal(np.sqrt(far).astype(F), ref[::97])
+
+
 @pytest.mark.parametrize("k", [1, 2, 8, 33, 64, 70, 200])
 @pytest.mark.parametrize("edge", [1.0, 1.25, 1.5, 1.75, 0.0625, 1.0625, 1.4375, 1.00390625])
 @pytest.mark.parametrize("shell", [0, 500])
@@ -49,17 +70,24 @@ def test_order_across_a_bin_edge(k, edge, shell):
         rad = np.sqrt(edge) * np.concatenate([r.uniform(0.1, 0.6, k - 1), r.uniform(1.01, 1.3, shell), [1.5]])
         xyz = np.concatenate([[q, a, b], (q + u * rad[:, None]).astype(F)]).astype(F)
         xyz = np.ascontiguousarray(xyz[r.permutation(len(xyz))])
-        idx = L.sf_build_index(torch.from_numpy(xyz).cuda())
-        try:
-            L.sf_bandwidths(idx, L.make_params(k=k))
-            h = torch.empty(len(xyz), device="cuda")
-            L.sf_get_bandwidths(idx, h)
-            nbr = torch.empty((len(xyz), k), dtype=torch.int32, device="cuda")
-            h2 = torch.empty_like(h)
-            L.sf_knn_neighbours(idx, k, nbr, h2)
-            torch.cuda.synchronize()
-        finally:
-            L.sf_free_index(idx)
-        ref = np.asarray(oracle.knn(xyz, k)[0], dtype=F)
-        assert np.array_equal(h.cpu().numpy().view(np.uint32), ref.view(np.uint32))
-        assert np.array_equal(h2.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+        _check(xyz, k)
+
+
+SCALES = {
+    # one point so far out that a scale chosen for it would push the others' squares to zero
+    "outlier": lambda r, n: np.concatenate([r.random((n - 1, 3)), [[1e30, 0.0, 0.0]]]),
+    "sentinel": lambda r, n: np.concatenate([r.random((n - 1, 3)), [[3e38, 3e38, 3e38]]]),
+    "close_pairs": lambda r, n: np.concatenate([1e-12 * r.random((n - 1, 3)), [[1e38, 0.0, 0.0]]]),
+    # one axis far from zero against the others' extent: a scale for the extent would overflow it
+    "plane": lambda r, n: np.concatenate([2.0 ** -100 * r.random((n, 2)), np.full((n, 1), 2.0)], axis=1),
+    "far_plane": lambda r, n: np.concatenate([1e-19 * r.random((n, 2)), np.full((n, 1), 1e30)], axis=1),
+    # no scale helps: squares among the smallest floats
+    "narrow": lambda r, n: np.concatenate([2.0 ** -64 * r.random((n, 2)), np.full((n, 1), 2.0 ** 126)], axis=1),
+}
+
+
+@pytest.mark.parametrize("cloud", sorted(SCALES))
+@pytest.mark.parametrize("k", [1, 8, 64, 100])
+def test_scales(cloud, k):
+    r = np.random.default_rng(k)
+    _check(SCALES[cloud](r, 1500)[r.permutation(1500)], k)
