@@ -694,9 +694,9 @@ __global__ void __launch_bounds__(kKnnWarps * 32, 7) k_knn(const __grid_constant
 //     evaluated again in FP32 (its d2 is good to 5 * 2^-24, far less than a code), and
 //     the k-th and what ties with it within 2e-6 in FP64, ranked by (d2, original
 //     index).
-// A leaf that this cannot resolve (more equal codes than a list holds, as among exact
-// duplicates; distances near the FP32 underflow; more than 1024 visited leaves) goes
-// to a retry list for the next kernel: longer lists, then k_knn.
+// A leaf that this cannot resolve (more equal codes than a list holds, more than 1024 visited
+// leaves) goes to a retry list for the same search with longer lists, then to k_knn; one
+// whose distances leave the FP32 range straight to k_knn.
 //
 // What bounds it: issue slots (43,000 instructions a leaf at k = 64, 55% of the slots at
 // the 10 warps an SM that the lists leave room for). 16.8M clustered points, k = 64,
@@ -734,8 +734,10 @@ struct KnnSelArgs {
     unsigned int *next_leaf;     // work counter (zeroed before launch)
     const unsigned int *todo;    // nullable: the query leaves to process (*todo_n of them)
     const unsigned int *todo_n;
-    unsigned int *retry;         // [leaves] the leaves left to the next kernel
+    unsigned int *retry;         // [leaves] the leaves left to the next kernel: longer lists
     unsigned int *retry_n;       // their number (zeroed before launch)
+    unsigned int *beyond;        // [leaves] those that FP32 distances cannot resolve: k_knn
+    unsigned int *beyond_n;
     unsigned long long *work;    // nullable: as KnnArgs::work
 };
 
@@ -749,7 +751,7 @@ struct KnnSel {
     float T;
     int cnt, seq;
     int head, staged;            // the ring: first staged candidate, how many (warp-uniform)
-    bool fail;                   // warp-uniform
+    bool fail, below32;          // warp-uniform: given up; because a k-th d2 is out of FP32's range
     float env_lo[3], env_hi[3];  // box around all lanes' balls
     unsigned long long ncand = 0;
 
@@ -1009,11 +1011,19 @@ struct KnnSel {
         } else {
             for (int i = 0; i < nmem; ++i)
                 S.list[CAP / 2 + i][lane] = __float_as_uint(d2_f32(q, __ldg(&tv.pos[point_of(S.list[i][lane])])));
-            for (int i = 0; i < nmem; ++i) {
-                const float di = __uint_as_float(S.list[CAP / 2 + i][lane]);
-                int le = 0;
-                for (int j = 0; j < nmem; ++j) le += __uint_as_float(S.list[CAP / 2 + j][lane]) <= di;
-                if (le >= need) dk = fminf(dk, di);
+            for (int le = 0; le < need && nmem > 0;) {  // from one value to the next
+                const float last = dk == INFINITY ? -1.f : dk;
+                float next = INFINITY;
+                int c = 0;
+                for (int i = 0; i < nmem; ++i) {
+                    const float di = __uint_as_float(S.list[CAP / 2 + i][lane]);
+                    if (di > last && di <= next) {
+                        c = di < next ? 1 : c + 1;
+                        next = di;
+                    }
+                }
+                dk = next;
+                le += max(c, 1);
             }
             for (int i = 0; i < nmem; ++i) {
                 const float di = __uint_as_float(S.list[CAP / 2 + i][lane]);
@@ -1027,32 +1037,40 @@ struct KnnSel {
         if (found && !(dk > 1.0e-34f && dk < 1.0e37f)) ok = false;
         if (found && ok) {
             kth = d2_f64(q, __ldg(&tv.pos[at]));
-            if (ties > 1) {  // rank them in FP64, by extraction
-                double last_d = -1.0;
-                uint32_t last_i = 0;
-                for (int left = need - sure; left > 0; --left) {
-                    double best_d = INFINITY;
-                    uint32_t best_i = 0xffffffffu;
+            if (ties > 1) {  // rank them in FP64, from one value to the next (exact ties are one)
+                kth = -1.0;
+                for (int left = need - sure; left > 0;) {
+                    double next = INFINITY;
+                    int c = 0;
                     for (int i = 0; i < nmem; ++i) {
                         const float di = __uint_as_float(S.list[CAP / 2 + i][lane]);
                         if (di < dk * (1.0f - kDelta) || di > dk * (1.0f + kDelta)) continue;
-                        const int j = point_of(S.list[i][lane]);
-                        const double dd = d2_f64(q, __ldg(&tv.pos[j]));
-                        const uint32_t id = __ldg(&a.perm[j]);
-                        if ((last_d < 0.0 || key_less(last_d, last_i, dd, id)) &&
-                            key_less(dd, id, best_d, best_i)) {
-                            best_d = dd;
-                            best_i = id;
+                        const double dd = d2_f64(q, __ldg(&tv.pos[point_of(S.list[i][lane])]));
+                        if (dd > kth && dd <= next) {
+                            c = dd < next ? 1 : c + 1;
+                            next = dd;
                         }
                     }
-                    last_d = best_d;
-                    last_i = best_i;
+                    kth = next;
+                    left -= max(c, 1);
                 }
-                kth = last_d;
             }
         }
-        fail = !__all_sync(0xffffffffu, ok);
+        fail = below32 = !__all_sync(0xffffffffu, ok);
         return kth;
+    }
+
+    // More than k points of the run around qi at its place? Points that coincide follow one another
+    // in the index (prev, next: whether the neighbours do).
+    __device__ bool coincide(int qi, bool prev, bool next) const {
+        auto same = [&](int i) {
+            const float4 p = __ldg(&a.tv.pos[i]);
+            return p.x == q.x && p.y == q.y && p.z == q.z;
+        };
+        int lo = qi, hi = qi;
+        while (prev && lo > 0 && hi - lo < a.k && same(lo - 1)) --lo;
+        while (next && hi + 1 < (int)a.tv.n && hi - lo < a.k && same(hi + 1)) ++hi;
+        return hi - lo >= a.k;
     }
 
     __device__ void leaf(int leaf) {
@@ -1060,10 +1078,29 @@ struct KnnSel {
         const TreeView &tv = a.tv;
         const int n_all = (int)tv.n, nleaf = (int)tv.cnt[0];  // both below 2^31
         const int qi = leaf * kLeaf + lane;
-        const bool valid = qi < n_all;
+        bool valid = qi < n_all;
         q = valid ? __ldg(&tv.pos[qi]) : make_float4(0.f, 0.f, 0.f, 0.f);
         cnt = seq = head = staged = 0;
-        fail = false;
+        fail = below32 = false;
+        // More than k points at one place: the k-th is at 0, which FP32 distances do not show (1M
+        // points at 25,000 places, k = 8: 12.2 ms when such leaves went to k_knn, 0.33 ms now).
+        // Where few warps hide the loads of the neighbours they are shuffled: k = 64 of 4M
+        // clustered points takes 1% longer with this, 3.5% by loads; k = 8 0% by loads, 2% so.
+        bool prev = true, next = true;
+        if (CAP > 128) {
+            const float4 o = __ldg(&tv.pos[lane == 0 ? max(qi - 1, 0) : min(qi + 1, n_all - 1)]);  // lanes 0 and 31
+            auto same = [&](float x, float y, float z, bool edge) {
+                return edge ? o.x == q.x && o.y == q.y && o.z == q.z : x == q.x && y == q.y && z == q.z;
+            };
+            prev = same(__shfl_up_sync(0xffffffffu, q.x, 1), __shfl_up_sync(0xffffffffu, q.y, 1),
+                        __shfl_up_sync(0xffffffffu, q.z, 1), lane == 0);
+            next = same(__shfl_down_sync(0xffffffffu, q.x, 1), __shfl_down_sync(0xffffffffu, q.y, 1),
+                        __shfl_down_sync(0xffffffffu, q.z, 1), lane == 31);
+        }
+        if (valid && (prev || next) && coincide(qi, prev, next)) {
+            a.h_sorted[qi] = 0.f;
+            valid = false;
+        }
         groups(valid);
 
         // ---- 1. the leaves around this one: any k of their points bound the k-th distance
@@ -1239,7 +1276,10 @@ struct KnnSel {
         double kth = 0.0;
         if (!fail) kth = kth_d2(valid);
         if (fail) {
-            if (lane == 0) a.retry[atomicAdd(a.retry_n, 1u)] = (unsigned int)leaf;
+            if (lane == 0) {
+                if (below32) a.beyond[atomicAdd(a.beyond_n, 1u)] = (unsigned int)leaf;
+                else a.retry[atomicAdd(a.retry_n, 1u)] = (unsigned int)leaf;
+            }
         } else if (valid) {
             a.h_sorted[qi] = (float)sqrt(kth);
         }
@@ -1361,9 +1401,10 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
         b.next_leaf = counters + 1;
         b.todo = b.todo_n = nullptr;
         b.retry_n = counters + 3;
-        b.retry = sc.get<unsigned int>(idx->cnt[0]);
+        b.retry = sc.get<unsigned int>(k <= 66 ? idx->cnt[0] : 1);
+        b.beyond_n = counters + 4;
+        b.beyond = sc.get<unsigned int>(idx->cnt[0]);
         b.work = d_work;
-        unsigned int *retry2 = sc.get<unsigned int>(idx->cnt[0]);
         SF_TRY_SCRATCH(sc);
         if (k <= 66) {
             if (k <= 34) SF_TRY((launch_sel<96, 13>(b, idx->cnt[0], sc, s)));
@@ -1372,8 +1413,8 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
             b.todo_n = b.retry_n;
         }
         b.next_leaf = counters + 2;
-        b.retry_n = counters + 4;
-        b.retry = retry2;
+        b.retry_n = b.beyond_n;
+        b.retry = b.beyond;
         SF_TRY((launch_sel<400, 4>(b, idx->cnt[0], sc, s)));
         a.retry = b.retry;
         a.retry_n = b.retry_n;

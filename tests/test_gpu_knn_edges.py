@@ -91,3 +91,21 @@ SCALES = {
 def test_scales(cloud, k):
     r = np.random.default_rng(k)
     _check(SCALES[cloud](r, 1500)[r.permutation(1500)], k)
+
+
+@pytest.mark.parametrize("k", [1, 8, 33, 64, 100])
+@pytest.mark.parametrize("each", [2, 9, 40, 60, 150])
+@pytest.mark.parametrize("apart", ["exact", "near", "lattice"])
+def test_coinciding(each, k, apart):
+    """Places that hold several points: the k-th at distance 0, among many at one distance, or
+    (near) at distances whose squares FP32 cannot tell from 0."""
+    r = np.random.default_rng(each + k)
+    n = 3000
+    at = r.integers(0, n // each, n)
+    if apart == "lattice":
+        p = np.stack([at % 7, at // 7 % 7, at // 49], axis=1) * 0.1
+    else:
+        p = r.random((n // each, 3))[at]
+    if apart == "near":
+        p[:, 2] = 1e-24 * r.integers(0, 3, n)
+    _check(p, k)
