@@ -10,8 +10,9 @@
 //
 // One thread per destination column of 8 nodes; a node's cell in the source grid and
 // its weights are formed in FP64 once per axis (the source grid's node coordinates as
-// lo + i s, like every grid of the library), the eight-point weighted sum in pairs
-// of floats (about 45 bits), one rounding to float at the end.
+// lo + i s, like every grid of the library). The eight-point weighted sum is that of FP64
+// rounded once to float: evaluated in pairs of floats, and again in FP64 where the pairs'
+// error leaves the rounding open.
 #include <cmath>
 
 #include "sf_internal.cuh"
@@ -44,13 +45,21 @@ __device__ __forceinline__ double axis_cell(const Axes &A, int k, int id, int &c
     return v - (double)c;
 }
 
-// Float pairs: s + e = a + b exactly (no ordering of |a| and |b| needed).
+// Float pairs: s + e = a + b exactly (Knuth's two-sum: no ordering of |a| and |b| needed).
 __device__ __forceinline__ float sum2(float a, float b, float &e) {
     const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
     return s;
 }
-// (ah + al) w0 + (bh + bl) w1 to about 45 bits.
+// a w0 + b w1 and (ah + al) w0 + (bh + bl) w1 in float pairs.
+__device__ __forceinline__ float mix1(float a, float b, const AxisPlace &p, float &lo) {
+    const float s = __fmul_rn(a, p.w0h), t = __fmul_rn(b, p.w1h);
+    const float es = fmaf(a, p.w0l, fmaf(a, p.w0h, -s)), et = fmaf(b, p.w1l, fmaf(b, p.w1h, -t));
+    float e;
+    const float r = sum2(s, t, e);
+    lo = e + (es + et);
+    return r;
+}
 __device__ __forceinline__ float mix2(float ah, float al, float bh, float bl, const AxisPlace &p, float &lo) {
     const float s = __fmul_rn(ah, p.w0h), t = __fmul_rn(bh, p.w1h);
     const float es = fmaf(al, p.w0h, fmaf(ah, p.w0l, fmaf(ah, p.w0h, -s)));
@@ -61,55 +70,62 @@ __device__ __forceinline__ float mix2(float ah, float al, float bh, float bl, co
     return r;
 }
 
-// The same in FP64: for nodes whose value leaves the range in which float pairs are exact.
-__device__ __noinline__ float resample_fp64(const float *__restrict__ src, const Axes &A, float weight, int ix,
-                                            int iy, int iz) {
-    const int id[3] = {ix, iy, iz};
-    double u[3];
-    int c[3];
-    bool in;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) u[k] = axis_cell(A, k, id[k], c[k], in);
+// The same in FP64, for nodes that the float pairs cannot settle.
+__device__ __noinline__ float resample_fp64(const float *__restrict__ f, int64_t row, int64_t slice, double ux,
+                                            double uy, double uz, float weight) {
+    const double vx = 1.0 - ux, vy = 1.0 - uy, vz = 1.0 - uz;
+    const double w[4] = {vx * vy, ux * vy, vx * uy, ux * uy};
     double val = 0.0;
-    for (int t = 0; t < 8; ++t) {
-        const int dx = t & 1, dy = (t >> 1) & 1, dz = t >> 2;
-        const double w = (dx ? u[0] : 1.0 - u[0]) * (dy ? u[1] : 1.0 - u[1]) * (dz ? u[2] : 1.0 - u[2]);
-        val += w * (double)__ldg(&src[((int64_t)(c[2] + dz) * A.n[1] + (c[1] + dy)) * A.n[0] + (c[0] + dx)]);
-    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+        val += w[t & 3] * (t >> 2 ? uz : vz) * (double)__ldg(f + (t & 1) + ((t >> 1) & 1) * row + (t >> 2) * slice);
     return (float)((double)weight * val);
 }
 
 // What bounds it: with every node's cell, weights and sum in FP64 (about 70 instructions
 // at 2 lanes a clock and SM) it ran at the FP64 rate: 108 us for 96^3 nodes. Per-axis
-// places (one FP64 evaluation per block and axis node) leave the sum, about 110 FP32
-// instructions in float pairs with the same error (the final rounding): 8.8 us, bounded
-// by issue and the blocks' start-up (7.4 MB of compulsory traffic would take 1.1 us).
-constexpr int kRsX = 32, kRsY = 8, kRsZ = 8;
+// places (one FP64 evaluation per block and axis node) leave the sum, about 120 FP32
+// instructions in float pairs: 8.8 us (11 with cold caches), bounded by issue and the blocks' start-up (7.4 MB of
+// compulsory traffic would take 1.1 us). Settling the rounding costs about 0.7 us of that (calls in a row: 10.25 and 10.9 us). The pairs are good to 2^-41.8 of a sum of
+// non-negative terms (2^-45.3, 2^-43.6 and 2^-42.9 for the three steps, whose low parts grow
+// to 2^-20.7; 2^-44.7 for the weight; 2^-48 a pair of weights); kRsError covers that and the
+// 2^-49 of FP64, so where both ends of the interval round to one float, FP64 rounds to
+// it too: all but about one node in 90,000.
+constexpr float kRsError = 0x1p-41f;
+// A block takes 256 columns, in x the next power of two of narrow grids and else 32 (with 32
+// always, 2 x 4096 x 1024 nodes of a signed field, all FP64, took 14.5 ms).
+constexpr int kRsThreads = 256, kRsZ = 8;
 
-__global__ void __launch_bounds__(kRsX * kRsY)
-    k_resample(const float *__restrict__ src, Axes A, float weight, int accumulate, float *__restrict__ dst,
+__global__ void __launch_bounds__(kRsThreads)
+    k_resample(const float *__restrict__ src, Axes A, int xlog, float weight, int accumulate, float *__restrict__ dst,
                unsigned long long *outside) {
-    __shared__ AxisPlace P[kRsX + kRsY + kRsZ];
-    const int tid = threadIdx.x;
-    const int g0[3] = {(int)blockIdx.x * kRsX, (int)blockIdx.y * kRsY, (int)blockIdx.z * kRsZ};
-    if (tid < kRsX + kRsY + kRsZ) {
-        const int k = tid < kRsX ? 0 : (tid < kRsX + kRsY ? 1 : 2);
-        const int i = g0[k] + tid - (k == 0 ? 0 : (k == 1 ? kRsX : kRsX + kRsY));
+    __shared__ AxisPlace P[kRsThreads];  // of the block's nodes in x, y and z
+    __shared__ double U[kRsThreads];     // their FP64 places in the cell
+    const int tid = threadIdx.x, bx = 1 << xlog, by = kRsThreads >> xlog;
+    const int g0[3] = {(int)blockIdx.x * bx, (int)blockIdx.y * by, (int)blockIdx.z * kRsZ};
+    if (tid < bx + by + kRsZ) {
+        const int k = tid < bx ? 0 : (tid < bx + by ? 1 : 2);
+        const int i = g0[k] + tid - (k == 0 ? 0 : (k == 1 ? bx : bx + by));
         AxisPlace p;
         bool in;
         const double u = axis_cell(A, k, i, p.c, in), v = 1.0 - u;
         if (!in) p.c = -1;
+        U[tid] = u;
         p.w0h = (float)v;
         p.w0l = (float)(v - (double)p.w0h);
         p.w1h = (float)u;
         p.w1l = (float)(u - (double)p.w1h);
+        // a node a rounding past the box's face, or so near a source node that its weight's
+        // pair could leave the normal range: FP64 (no test of the sum passes a NaN)
+        // (1 - u is 0 or at least 2^-53; the high word of u is 0 for u = 0)
+        if (p.w0h < 0.f || (p.w1h < 0x1p-64f && __double2hiint(u) != 0)) p.w0h = NAN;
         P[tid] = p;
     }
     __syncthreads();
-    const int ix = g0[0] + (tid & (kRsX - 1)), iy = g0[1] + tid / kRsX;
+    const int ix = g0[0] + (tid & (bx - 1)), iy = g0[1] + (tid >> xlog);
     unsigned long long out_cnt = 0;
     if (ix < A.dn[0] && iy < A.dn[1]) {
-        const AxisPlace px = P[tid & (kRsX - 1)], py = P[kRsX + tid / kRsX];
+        const AxisPlace px = P[tid & (bx - 1)], py = P[bx + (tid >> xlog)];
         const int nz = min(kRsZ, A.dn[2] - g0[2]);
         const int64_t row = A.n[0], slice = (int64_t)A.n[0] * A.n[1];
         float *d = dst + ((int64_t)g0[2] * A.dn[1] + iy) * A.dn[0] + ix;
@@ -117,7 +133,7 @@ __global__ void __launch_bounds__(kRsX * kRsY)
         const float zero = weight * 0.f;  // a negative weight's zero is -0
 #pragma unroll 2
         for (int z = 0; z < nz; ++z) {
-            const AxisPlace pz = P[kRsX + kRsY + z];
+            const AxisPlace &pz = P[bx + by + z];
             float res = zero;
             if (px.c >= 0 && py.c >= 0 && pz.c >= 0) {
                 const float *f = src + pz.c * slice + py.c * row + px.c;
@@ -126,21 +142,27 @@ __global__ void __launch_bounds__(kRsX * kRsY)
                 const float f001 = __ldg(f + slice), f101 = __ldg(f + slice + 1);
                 const float f011 = __ldg(f + slice + row), f111 = __ldg(f + slice + row + 1);
                 float l00, l10, l01, l11, l0, l1, lo;
-                const float h00 = mix2(f000, 0.f, f100, 0.f, px, l00), h10 = mix2(f010, 0.f, f110, 0.f, px, l10);
-                const float h01 = mix2(f001, 0.f, f101, 0.f, px, l01), h11 = mix2(f011, 0.f, f111, 0.f, px, l11);
+                const float h00 = mix1(f000, f100, px, l00), h10 = mix1(f010, f110, px, l10);
+                const float h01 = mix1(f001, f101, px, l01), h11 = mix1(f011, f111, px, l11);
                 const float h0 = mix2(h00, l00, h10, l10, py, l0), h1 = mix2(h01, l01, h11, l11, py, l1);
                 const float hi = mix2(h0, l0, h1, l1, pz, lo);
                 const float r = __fmul_rn(weight, hi);
-                res = r + fmaf(weight, lo, fmaf(weight, hi, -r));
+                const float tail = fmaf(weight, lo, fmaf(weight, hi, -r)), err = kRsError * fabsf(r);
+                res = r + (tail + err);
                 const uint32_t any = __float_as_uint(f000) | __float_as_uint(f100) | __float_as_uint(f010) |
                                      __float_as_uint(f110) | __float_as_uint(f001) | __float_as_uint(f101) |
                                      __float_as_uint(f011) | __float_as_uint(f111);
-                // FP64 where a negative value may cancel others or a partial product may have
-                // left the normal range (infinities and NaN among them); all-zero neighbours
-                // are exact
-                const bool plain = (int)any >= 0 && fabsf(hi) > 1.0e-28f && fabsf(hi) < 1.0e37f &&
-                                   ((fabsf(r) > 1.0e-28f && fabsf(r) < 1.0e37f) || weight == 0.f);
-                if (!plain) res = any ? resample_fp64(src, A, weight, ix, iy, g0[2] + z) : zero;
+                // FP64 where the rounding is open, a negative value may cancel others or a partial
+                // product may have left the normal range (infinities and NaN among them);
+                // all-zero neighbours and a weight of 0 are exact
+                bool plain = (int)any >= 0 && hi > 1.0e-28f && hi < 1.0e37f && fabsf(r) > 1.0e-28f && fabsf(r) < 1.0e37f &&
+                             res == r + (tail - err);
+                if (any == 0 || (weight == 0.f && (int)any > 0 && hi < 1.0e37f)) {
+                    res = zero;
+                    plain = true;
+                }
+                if (!plain)
+                    res = resample_fp64(f, row, slice, U[tid & (bx - 1)], U[bx + (tid >> xlog)], U[bx + by + z], weight);
             } else {
                 ++out_cnt;
             }
@@ -194,8 +216,11 @@ extern "C" sf_status sf_resample_grid(const float *d_src, const sf_box *src_box,
         SF_TRY_SCRATCH(sc);
         SF_TRY_CUDA(cudaMemsetAsync(cnt, 0, sizeof *cnt, s));
     }
-    const dim3 grid((A.dn[0] + kRsX - 1) / kRsX, (A.dn[1] + kRsY - 1) / kRsY, (A.dn[2] + kRsZ - 1) / kRsZ);
-    SF_TRY_CUDA(launch(k_resample, grid, dim3(kRsX * kRsY), 0, s, d_src, A, weight, accumulate ? 1 : 0, d_dst, cnt));
+    int xlog = 1;
+    while (xlog < 5 && (1 << xlog) < A.dn[0]) ++xlog;
+    const int bx = 1 << xlog, by = kRsThreads >> xlog;
+    const dim3 grid((A.dn[0] + bx - 1) / bx, (A.dn[1] + by - 1) / by, (A.dn[2] + kRsZ - 1) / kRsZ);
+    SF_TRY_CUDA(launch(k_resample, grid, dim3(kRsThreads), 0, s, d_src, A, xlog, weight, accumulate ? 1 : 0, d_dst, cnt));
     if (h_outside) {
         unsigned long long h = 0;
         SF_TRY_CUDA(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, s));

@@ -1,6 +1,8 @@
 """sf_resample_grid and sf_iso_surface at the edges of their kernels: ragged and smallest
 grids, nodes on the source box's faces, values that leave the range of the fast paths
 (negative, tiny, huge, infinite, NaN, zero), weights and thresholds out of the ordinary."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -111,3 +113,57 @@ def test_iso_with_infinities():
     inside = grid > 0.5
     corner = [[0, 1, 3, 7], [0, 1, 5, 7], [0, 2, 3, 7], [0, 2, 6, 7], [0, 4, 5, 7], [0, 4, 6, 7]]
     assert n == sum({0: 0, 4: 0, 2: 2}.get(int(inside[c].sum()), 1) for c in corner)
+
+
+@pytest.mark.parametrize("dst,weight", [((400, 400, 400), 1.0), ((512, 256, 192), 0.7), ((2, 1000, 3000), 1.0),
+                                        ((3, 1001, 2000), -3.3), ((17, 900, 700), 1.0)])
+def test_resample_is_the_fp64_sum_rounded_once(dst, weight):
+    """Every node is the FP64 sum (one fused step a neighbour) rounded to float. Where the
+    interval of 2^-43 around it rounds to one float that one; the others are summed again in
+    rationals, rounded to FP64 at each step."""
+    g = torch.Generator(device="cuda").manual_seed(7)
+    dims, box = (61, 67, 59), ((0.0, -1.0, 2.0), (1.0, 1.0, 7.0))
+    src = torch.exp(2.0 * torch.randn(dims[::-1], generator=g, device="cuda"))
+    dst_box = ((0.0, -0.9, 2.1), (1.0, 1.0, 6.3))
+    out = torch.empty(dst[::-1], device="cuda")
+    L.sf_resample_grid(src.reshape(-1), L.make_box(*box), dims, L.make_box(*dst_box), dst, out, weight=weight)
+    f, cell, u = src.double(), [], []
+    for k in range(3):
+        s = (box[1][k] - box[0][k]) / (dims[k] - 1)
+        r = dst_box[0][k] + torch.arange(dst[k], device="cuda", dtype=torch.float64) * (
+            (dst_box[1][k] - dst_box[0][k]) / (dst[k] - 1))
+        v = (r - box[0][k]) * (1.0 / s)
+        cell.append(v.floor().long().clamp(0, dims[k] - 2))
+        u.append(v - cell[k])
+    w32 = float(np.float32(weight))
+    open_nodes = []
+    for z in range(dst[2]):
+        val = torch.zeros((dst[1], dst[0]), device="cuda", dtype=torch.float64)
+        for dz in range(2):
+            plane, wz = f[cell[2][z] + dz], (u[2][z] if dz else 1 - u[2][z])
+            for dy in range(2):
+                for dx in range(2):
+                    w = (u[0] if dx else 1 - u[0])[None, :] * (u[1] if dy else 1 - u[1])[:, None] * wz
+                    val += w * plane[cell[1] + dy][:, cell[0] + dx]
+        val *= w32
+        lo, hi = (val * (1 - 2.0 ** -43)).float(), (val * (1 + 2.0 ** -43)).float()
+        assert bool(((out[z] == lo) | (lo != hi)).all())
+        open_nodes += [(z, int(y), int(x)) for y, x in torch.nonzero(lo != hi).tolist()]
+    assert dst[0] < 400 or len(open_nodes) > 20
+    fc, uc, cc = src.cpu().numpy(), [a.cpu().tolist() for a in u], [a.cpu().tolist() for a in cell]
+    for z, y, x in open_nodes:
+        val = 0.0
+        for t in range(8):
+            dx, dy, dz = t & 1, t >> 1 & 1, t >> 2
+            w = (uc[0][x] if dx else 1.0 - uc[0][x]) * (uc[1][y] if dy else 1.0 - uc[1][y])
+            w *= uc[2][z] if dz else 1.0 - uc[2][z]
+            val = float(Fraction(w) * Fraction(float(fc[cc[2][z] + dz, cc[1][y] + dy, cc[0][x] + dx])) + Fraction(val))
+        assert float(out[z, y, x]) == float(np.float32(w32 * val)), (z, y, x)
+
+
+def test_resample_weight_of_negative_zero():
+    out = torch.full((4 * 4 * 4,), 7.0, device="cuda")
+    L.sf_resample_grid(torch.ones(27, device="cuda"), L.make_box((0, 0, 0), (1, 1, 1)), (3, 3, 3),
+                       L.make_box((0, 0, 0), (1, 1, 1)), (4, 4, 4), out, weight=-0.0)
+    got = out.cpu().numpy()
+    assert not got.any() and np.signbit(got).all()
