@@ -2122,9 +2122,11 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
     }
     // A leaf whose points lie apart (at a jump of the Morton order) has a box that can cover
     // clusters none of its points is near: from kWideLeaves candidate leaves on (the mean is
-    // about 200) nodes and candidates are tested against every point. A whole launch
-    // waited for single such leaves, of up to 36,000 candidate leaves: the densities at
-    // 16.8M clustered points took 44.2 ms, 23.6 ms with this test.
+    // about 200) nodes are tested against every point. A whole launch waited for single
+    // such leaves, of up to 36,000 candidate leaves: the densities at 16.8M clustered
+    // points took 44.2 ms, 23.6 ms with this test. (Testing the candidates themselves so costs
+    // what it saves there, and where every leaf is wide, as with the estimator's long
+    // lengths, 1.7 times the whole: 4M points over the cube 1.43 s, 0.86 s without.)
     bool wide = false;
     int seen = 0;
     S.q[lane] = make_float4(active ? q.x : INFINITY, q.y, q.z, 0.f);
@@ -2252,15 +2254,6 @@ __global__ void __launch_bounds__(kPtWarps * 32) k_points(PointsArgs a) {
                     qlb = fmaf(t, t, qlb);
                 }
                 ok = ok && qlb < KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
-                if (wide && ok) {
-                    ok = false;
-                    for (int e = 0; e < kLeaf; ++e) {
-                        const float4 w = S.q[e];
-                        const float tx = (w.x - p.x) * r[0], ty = (w.y - p.y) * r[1], tz = (w.z - p.z) * r[2];
-                        ok = ok || fmaf(tz, tz, fmaf(ty, ty, tx * tx)) <
-                                       KDef<KER>::rmul * KDef<KER>::rmul * (1.0f + kFilterSlack);
-                    }
-                }
             }
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok) {
