@@ -923,16 +923,21 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
         }
         __syncwarp();
         float mcen[3], mhw[3];  // the tile box widened by the rounding margin, as centre and half-width
-        float sp3[3];           // node spacing
+        // node spacing (of the float pairs: it may lie below the coordinates' float rounding); 0 on
+        // all axes where the pairs themselves are too coarse to tell the nearest node from it
+        float sp3[3];
+        bool even = true;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int off = k == 0 ? 0 : (k == 1 ? kWX : kWX + kWY);
             const float lo = S.axt[off].x, hi = S.axt[off + nv[k] - 1].x;
-            sp3[k] = nv[k] > 1 ? S.axt[off + 1].x - lo : 0.f;
+            sp3[k] = nv[k] > 1 ? (S.axt[off + 1].x - lo) + (S.axt[off + 1].y - S.axt[off].y) : 0.f;
+            even = even && (nv[k] == 1 || sp3[k] > 0x1p-44f * fmaxf(fabsf(lo), fabsf(hi)));
             const float mg = 1.0e-6f * (fabsf(lo) + fabsf(hi));
             mcen[k] = 0.5f * ((lo - mg) + (hi + mg));
             mhw[k] = 0.5f * ((hi + mg) - (lo - mg));
         }
+        if (!even) sp3[0] = sp3[1] = sp3[2] = 0.f;
         float acc[TZ], sum[TZ], cmp[TZ];
 #pragma unroll
         for (int k = 0; k < TZ; ++k) acc[k] = sum[k] = cmp[k] = 0.f;
@@ -987,7 +992,7 @@ __global__ void __launch_bounds__(kGridThreads, BW == BW_ANISO ? 3 : 4)
                         for (int k = 0; k < 3; ++k) {
                             const int off = k == 0 ? 0 : (k == 1 ? kWX : kWX + kWY);
                             const float u = KDef<KER>::uscale * rl[k];
-                            const float at = sp3[k] > 0.f ? (pc[k] - S.axt[off].x) / sp3[k] : 0.f;
+                            const float at = sp3[k] > 0.f ? ((pc[k] - S.axt[off].x) - S.axt[off].y) / sp3[k] : 0.f;
                             const int ic = (int)rintf(fminf(fmaxf(at, 0.f), (float)(nv[k] - 1)));
                             float m = INFINITY;
 #pragma unroll

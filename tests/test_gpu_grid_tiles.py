@@ -85,3 +85,39 @@ def test_grid_tiles(dims, n, kernel, reach):
             o = o.cpu().numpy().astype(np.float64)
             _check(o, ref, f"batch {dims} {n} {kernel} {reach}")
             assert abs(mm - o.sum() * cell) <= 1e-12 * abs(mm)
+
+
+@pytest.mark.parametrize("kernel", ["GAUSS3", "EPAN"])
+@pytest.mark.parametrize("far,width", [(1.0e6, 0.5), (1.0e6, 2.0), (3.0e4, 0.01), (1.0e6, 1.0e-6), (0.0, 0.5)])
+def test_node_spacing_below_the_coordinates_rounding(kernel, far, width):
+    """A box so narrow in x, so far out, that neighbouring nodes share their nearest float;
+    supports below the node spacing in z, of some steps of the coordinates in x."""
+    r = np.random.default_rng(int(far) + len(kernel))
+    n, dims = 3000, (40, 21, 6)
+    ulp = float(np.spacing(np.float32(far + width)))
+    xyz = r.random((n, 3)) * np.array([0.0, 10.0, 10.0])
+    xyz[:, 0] = far + max(ulp, width / 40) * r.integers(-4, 12, n)
+    xyz = xyz.astype(np.float32)
+    box = ((far, 0.0, 0.0), (far + width, 10.0, 10.0))
+    f = 3.0 if kernel == "GAUSS3" else 1.0
+    lengths = (2.3 * max(ulp, width / 40) / f, 0.9 / f, 0.9 / f)
+    p = _params("fixed", 8, lengths, "GLOBAL")
+    idx = L.sf_build_index(torch.from_numpy(xyz).cuda())
+    ker, nodes = getattr(L, "SF_K_" + kernel), dims[0] * dims[1] * dims[2]
+    try:
+        L.sf_bandwidths(idx, p)
+        outs = [torch.empty(nodes, device="cuda") for _ in range(3)]
+        L.sf_kde_grid(idx, L.make_box(*box), dims, ker, p, outs[0])
+        for z, o in ((4, outs[1]), (8, outs[2])):
+            t = L.sf_tune()
+            t.tile_z = z
+            b = L.sf_batch_create(idx, [L.make_box(*box)], [dims], ker, p, tune=t)
+            L.sf_batch_run(b, [o])
+            torch.cuda.synchronize()
+            L.sf_batch_free(b)
+    finally:
+        L.sf_free_index(idx)
+    ell = np.tile(np.float32(lengths).astype(np.float64), (n, 1))
+    ref = oracle.kde_grid(xyz, ell, box, dims, getattr(oracle, kernel), oracle.SCOPE_GLOBAL)
+    for o in outs:
+        _check(o.cpu().numpy().astype(np.float64), ref, f"{kernel} {far} {width}")
