@@ -347,8 +347,8 @@ __device__ __forceinline__ int tet_triangles(const IsoGrid &G, const float *__re
     return ntri;
 }
 
-// A block takes kIsoCells consecutive cells (x fastest), a warp 256 of them in 8 steps of
-// 32. A cell is first only the 8-bit mask of its corners above the threshold: (double)f > t
+// A warp takes 32 STEPS consecutive cells (x fastest) in STEPS steps of 32, a block those of
+// its eight warps. A cell is first only the 8-bit mask of its corners above the threshold: (double)f > t
 // exactly when f > the largest float up to t, so no FP64 is needed to count. Count
 // pass: the block's triangles. Emit pass (blocks with any): the warps' cut tetrahedra
 // are queued in shared memory and worked off 32 at a time, so that FP64 runs
@@ -357,9 +357,12 @@ __device__ __forceinline__ int tet_triangles(const IsoGrid &G, const float *__re
 // passes and the few cut cells of a warp on their own lanes, 192^3 nodes and 0.85
 // million triangles took 4.5 ms (FP64 and divergence): 0.03 ms to count and 0.34 ms to
 // emit now, still FP64 (a division, six products and the orientation a crossing).
+//
+// STEPS is 8, and 1 below four blocks of 8 an SM: there a warp's chain of FP64 batches sets the
+// time (16^3 nodes of noise, five cut tetrahedra a cell: 580 us a call with 8, 125 with 1).
 constexpr int kIsoWarps = 8;
 constexpr int kIsoSteps = 8;
-constexpr int kIsoCells = kIsoWarps * kIsoSteps * 32;
+constexpr int kIsoSmall = 4 * 152;  // blocks of 8 steps below which a warp takes one step
 
 // Bit c of a tetrahedron's mask = corner c of the cell (x | y << 1 | z << 2).
 __device__ __forceinline__ int tet_mask(int o) {
@@ -407,6 +410,7 @@ __device__ __forceinline__ void iso_table(uint16_t *table) {
     __syncthreads();
 }
 
+template <int STEPS>
 __global__ void __launch_bounds__(kIsoWarps * 32)
     k_iso_count(const float *__restrict__ grid, IsoGrid G, int64_t nc, uint32_t *__restrict__ cnt) {
     __shared__ uint16_t table[256];
@@ -414,10 +418,10 @@ __global__ void __launch_bounds__(kIsoWarps * 32)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     iso_table(table);
     uint32_t t = 0;
-    const int64_t c0 = (int64_t)blockIdx.x * kIsoCells + warp * (kIsoSteps * 32) + lane;
+    const int64_t c0 = ((int64_t)blockIdx.x * kIsoWarps + warp) * (STEPS * 32) + lane;
     int cx, cy, cz;
 #pragma unroll 2
-    for (int s = 0; s < kIsoSteps; ++s) t += table[cell_mask(G, grid, c0 + 32 * s, nc, cx, cy, cz)] & 255u;
+    for (int s = 0; s < STEPS; ++s) t += table[cell_mask(G, grid, c0 + 32 * s, nc, cx, cy, cz)] & 255u;
     t = __reduce_add_sync(0xffffffffu, t);
     if (lane == 0) wsum[warp] = t;
     __syncthreads();
@@ -433,6 +437,7 @@ struct IsoWarpSmem {
     float tri[32 * 18];           // the triangles of 32 tetrahedra
 };
 
+template <int STEPS>
 __global__ void __launch_bounds__(kIsoWarps * 32)
     k_iso_emit(const float *__restrict__ grid, IsoGrid G, int64_t nc, const uint32_t *__restrict__ cnt,
                const uint32_t *__restrict__ off, float *__restrict__ tris) {
@@ -443,12 +448,12 @@ __global__ void __launch_bounds__(kIsoWarps * 32)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     iso_table(table);
-    const int64_t w0 = (int64_t)blockIdx.x * kIsoCells + warp * (kIsoSteps * 32);
-    unsigned mask[kIsoSteps];
+    const int64_t w0 = ((int64_t)blockIdx.x * kIsoWarps + warp) * (STEPS * 32);
+    unsigned mask[STEPS];
     uint32_t t = 0;
     int cx, cy, cz;
 #pragma unroll
-    for (int s = 0; s < kIsoSteps; ++s) {
+    for (int s = 0; s < STEPS; ++s) {
         mask[s] = cell_mask(G, grid, w0 + 32 * s + lane, nc, cx, cy, cz);
         t += table[mask[s]] & 255u;
     }
@@ -475,10 +480,10 @@ __global__ void __launch_bounds__(kIsoWarps * 32)
         __syncwarp();
     };
 #pragma unroll 1
-    for (int s = 0; s < kIsoSteps; ++s) {
+    for (int s = 0; s < STEPS; ++s) {
         unsigned m = 0;
 #pragma unroll
-        for (int k = 0; k < kIsoSteps; ++k)
+        for (int k = 0; k < STEPS; ++k)
             if (k == s) m = mask[k];
         const int cuts = table[m] >> 8;
         int before = cuts;  // inclusive scan over the lanes
@@ -533,13 +538,15 @@ extern "C" sf_status sf_iso_surface(const float *d_grid, const sf_box *roi, cons
     if ((double)G.tf > threshold) G.tf = nextafterf(G.tf, -INFINITY);
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t nc = (int64_t)(G.n[0] - 1) * (G.n[1] - 1) * (G.n[2] - 1);
-    const int64_t nb = (nc + kIsoCells - 1) / kIsoCells;
+    const bool small = nc < (int64_t)kIsoSmall * kIsoWarps * kIsoSteps * 32;
+    const int64_t cells = kIsoWarps * 32 * (small ? 1 : kIsoSteps), nb = (nc + cells - 1) / cells;
     Scratch sc(s);
     uint32_t *cnt = sc.get<uint32_t>(nb);
     uint32_t *off = sc.get<uint32_t>(nb);
     uint32_t *tot = sc.get<uint32_t>(1);
     SF_TRY_SCRATCH(sc);
-    SF_TRY_CUDA(launch(k_iso_count, dim3((unsigned)nb), dim3(kIsoWarps * 32), 0, s, d_grid, G, nc, cnt));
+    SF_TRY_CUDA(launch(small ? k_iso_count<1> : k_iso_count<kIsoSteps>, dim3((unsigned)nb), dim3(kIsoWarps * 32), 0, s,
+                       d_grid, G, nc, cnt));
     SF_TRY(scan_u32(cnt, off, nb, tot, s));
     uint32_t h = 0;
     SF_TRY_CUDA(cudaMemcpyAsync(&h, tot, sizeof h, cudaMemcpyDeviceToHost, s));
@@ -550,7 +557,7 @@ extern "C" sf_status sf_iso_surface(const float *d_grid, const sf_box *roi, cons
         return fail(SF_ERR_CAPACITY, "sf_iso_surface: %u triangles exceed capacity %lld", h, (long long)capacity);
     }
     if (h > 0)
-        SF_TRY_CUDA(launch(k_iso_emit, dim3((unsigned)nb), dim3(kIsoWarps * 32), 0, s, d_grid, G, nc,
-                           (const uint32_t *)cnt, (const uint32_t *)off, d_tris));
+        SF_TRY_CUDA(launch(small ? k_iso_emit<1> : k_iso_emit<kIsoSteps>, dim3((unsigned)nb), dim3(kIsoWarps * 32), 0, s,
+                           d_grid, G, nc, (const uint32_t *)cnt, (const uint32_t *)off, d_tris));
     return SF_OK;
 }

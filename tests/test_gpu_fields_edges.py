@@ -107,6 +107,28 @@ def test_iso_edges(dims, t):
         assert not short.any()
 
 
+@pytest.mark.parametrize("dims", [(131, 127, 83), (3, 700, 900), (1100, 2, 1200)])
+def test_iso_large_grid_is_its_slabs(dims):
+    """A grid large enough for the longer steps of a warp against slabs of it, which take single
+    ones (and which test_iso_edges compares with the oracle): the same triangles in order, up
+    to the rounding of the slabs' node coordinates."""
+    g = torch.Generator(device="cuda").manual_seed(dims[0])
+    f = torch.rand(dims[::-1], generator=g, device="cuda")
+    cap = 12 * (dims[0] - 1) * (dims[1] - 1) * (dims[2] - 1)
+    t, tris = 0.97, torch.zeros((cap // 4, 9), device="cuda")
+    n = L.sf_iso_surface(f.reshape(-1), L.make_box((0, 0, 0), tuple(float(d - 1) for d in dims)), dims, t, tris)
+    at = 0
+    for z in range(0, dims[2] - 1, 21):
+        m = min(22, dims[2] - z)
+        part = torch.zeros((cap // 4, 9), device="cuda")
+        c = L.sf_iso_surface(f[z:z + m].reshape(-1).contiguous(),
+                             L.make_box((0, 0, z), (float(dims[0] - 1), float(dims[1] - 1), float(z + m - 1))),
+                             (dims[0], dims[1], m), t, part)
+        assert torch.allclose(tris[at:at + c], part[:c], rtol=2.0 ** -22, atol=0.0)
+        at += c
+    assert at == n > 10_000 and not tris[n:].any()
+
+
 def test_iso_with_infinities():
     grid = np.array([0.0, 1.0, np.inf, -np.inf, 0.0, 1.0, np.nan, 2.0], dtype=np.float32)
     n = L.sf_iso_surface(torch.from_numpy(grid).cuda(), L.make_box((0, 0, 0), (1, 1, 1)), (2, 2, 2), 0.5)
