@@ -92,18 +92,22 @@ __device__ __noinline__ float resample_fp64(const float *__restrict__ f, int64_t
 // 2^-49 of FP64, so where both ends of the interval round to one float, FP64 rounds to
 // it too: all but about one node in 90,000.
 constexpr float kRsError = 0x1p-41f;
-// A block takes 256 columns, in x the next power of two of narrow grids and else 32 (with 32
-// always, 2 x 4096 x 1024 nodes of a signed field, all FP64, took 14.5 ms).
+// A block takes 256 columns of up to 8 nodes. A warp is 32 nodes wide in x, or narrower (8, in
+// grids narrower than that 2) where an eighth fewer warps cover the grid so (2 x 4096 x 1024
+// nodes of a signed field, all FP64: 14.5 ms with 32 always, 0.57 now; 33 x 300 x 300: 397
+// us and 260). Columns are shorter where the blocks would not fill the chip (33^3 nodes of a signed
+// field: 41 us a call with 8, 26 now).
 constexpr int kRsThreads = 256, kRsZ = 8;
+constexpr int kRsBlocks = 2 * 152;
 
 __global__ void __launch_bounds__(kRsThreads)
-    k_resample(const float *__restrict__ src, Axes A, int xlog, float weight, int accumulate, float *__restrict__ dst,
+    k_resample(const float *__restrict__ src, Axes A, int xlog, int zlen, float weight, int accumulate, float *__restrict__ dst,
                unsigned long long *outside) {
     __shared__ AxisPlace P[kRsThreads];  // of the block's nodes in x, y and z
     __shared__ double U[kRsThreads];     // their FP64 places in the cell
     const int tid = threadIdx.x, bx = 1 << xlog, by = kRsThreads >> xlog;
-    const int g0[3] = {(int)blockIdx.x * bx, (int)blockIdx.y * by, (int)blockIdx.z * kRsZ};
-    if (tid < bx + by + kRsZ) {
+    const int g0[3] = {(int)blockIdx.x * bx, (int)blockIdx.y * by, (int)blockIdx.z * zlen};
+    if (tid < bx + by + zlen) {
         const int k = tid < bx ? 0 : (tid < bx + by ? 1 : 2);
         const int i = g0[k] + tid - (k == 0 ? 0 : (k == 1 ? bx : bx + by));
         AxisPlace p;
@@ -126,7 +130,7 @@ __global__ void __launch_bounds__(kRsThreads)
     unsigned long long out_cnt = 0;
     if (ix < A.dn[0] && iy < A.dn[1]) {
         const AxisPlace px = P[tid & (bx - 1)], py = P[bx + (tid >> xlog)];
-        const int nz = min(kRsZ, A.dn[2] - g0[2]);
+        const int nz = min(zlen, A.dn[2] - g0[2]);
         const int64_t row = A.n[0], slice = (int64_t)A.n[0] * A.n[1];
         float *d = dst + ((int64_t)g0[2] * A.dn[1] + iy) * A.dn[0] + ix;
         const int64_t dslice = (int64_t)A.dn[0] * A.dn[1];
@@ -216,11 +220,15 @@ extern "C" sf_status sf_resample_grid(const float *d_src, const sf_box *src_box,
         SF_TRY_SCRATCH(sc);
         SF_TRY_CUDA(cudaMemsetAsync(cnt, 0, sizeof *cnt, s));
     }
-    int xlog = 1;
-    while (xlog < 5 && (1 << xlog) < A.dn[0]) ++xlog;
-    const int bx = 1 << xlog, by = kRsThreads >> xlog;
-    const dim3 grid((A.dn[0] + bx - 1) / bx, (A.dn[1] + by - 1) / by, (A.dn[2] + kRsZ - 1) / kRsZ);
-    SF_TRY_CUDA(launch(k_resample, grid, dim3(kRsThreads), 0, s, d_src, A, xlog, weight, accumulate ? 1 : 0, d_dst, cnt));
+    auto ceil_div = [](int n, int d) { return (n + d - 1) / d; };
+    auto warps = [&](int lg) { return (int64_t)ceil_div(A.dn[0], 1 << lg) * ceil_div(A.dn[1], 32 >> lg); };
+    int xlog = 5, zlen = kRsZ;
+    for (int lg = 4; lg >= (A.dn[0] < 8 ? 1 : 3); --lg)
+        if (8 * warps(lg) <= 7 * warps(xlog)) xlog = lg;
+    const int bx = ceil_div(A.dn[0], 1 << xlog), by = ceil_div(A.dn[1], kRsThreads >> xlog);
+    while (zlen > 1 && (int64_t)bx * by * ceil_div(A.dn[2], zlen) < kRsBlocks) zlen /= 2;
+    const dim3 grid(bx, by, ceil_div(A.dn[2], zlen));
+    SF_TRY_CUDA(launch(k_resample, grid, dim3(kRsThreads), 0, s, d_src, A, xlog, zlen, weight, accumulate ? 1 : 0, d_dst, cnt));
     if (h_outside) {
         unsigned long long h = 0;
         SF_TRY_CUDA(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, s));

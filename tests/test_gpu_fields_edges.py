@@ -189,3 +189,12 @@ def test_resample_weight_of_negative_zero():
                        L.make_box((0, 0, 0), (1, 1, 1)), (4, 4, 4), out, weight=-0.0)
     got = out.cpu().numpy()
     assert not got.any() and np.signbit(got).all()
+
+
+@pytest.mark.parametrize("field", ["density", "signed"])
+@pytest.mark.parametrize("dst", [(33, 40, 21), (5, 300, 9), (7, 33, 2), (9, 64, 64), (17, 130, 40), (97, 61, 3),
+                                 (65, 200, 120), (2, 129, 17), (4096, 2, 2)])
+def test_resample_block_shapes(field, dst):
+    """Grids on either side of the rules that shape a block: narrow, just wider than a warp's 8 or
+    32 nodes, few columns, few nodes in z."""
+    test_resample_edges(field, (19, 23, 29), dst, 1.0)
