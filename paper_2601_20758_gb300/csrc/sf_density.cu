@@ -1525,7 +1525,10 @@ static sf_status mr_sizes(const MrArgs &a, uint32_t total, int items_per_slot, i
     *slots = (int64_t)sms * per_sm;  // resident blocks of 8 persistent warps
     const int64_t warps = *slots * (kGridThreads / 32);
     const int64_t ips = std::max(1, items_per_slot);
-    *lpw = (uint32_t)std::max<int64_t>(16, (total + ips * warps - 1) / (ips * warps));
+    // At least 16 leaves an item (full staging passes), 8 where so few items leave warps without one:
+    // 24^3 nodes, fixed lengths, in 0.03 of a cloud of 4M points 203 us with 16, 194 with 8.
+    const int64_t least = total < 8 * warps ? 8 : 16;
+    *lpw = (uint32_t)std::max<int64_t>(least, (total + ips * warps - 1) / (ips * warps));
     *max_items = a.ntiles + total / *lpw + 1;
     return SF_OK;
 }
