@@ -1391,7 +1391,10 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
     if (!d_nbr_orig) {  // the neighbour ids are k_knn's
         // Lists of CAP entries: between leaves CAP - 32 of them, which have to hold k and the
         // boundary's ties and leave room, so that few leaves force a compaction; shared
-        // memory (128 bytes a row and warp) sets how many warps an SM holds.
+        // memory (128 bytes a row and warp) sets how many warps an SM holds. 144 entries serve up
+        // to k = 92: there 1M uniform points take 3.2 ms (400 entries 5.4), at 100 4.4 and 5.5,
+        // but 100,000 clustered ones 0.59 and 0.66, 0.83 and 0.68 ms (k_knn alone 8.3 and 7.2 ms,
+        // 2.4 and 2.5; with the line at 66, k = 67 took 4.90 ms, more than k_knn's 4.27).
         KnnSelArgs b;
         b.tv = a.tv;
         b.perm = a.perm;
@@ -1401,12 +1404,12 @@ sf_status knn_run(sf_index *idx, int k, uint32_t *d_nbr_orig, float *d_h_sorted,
         b.next_leaf = counters + 1;
         b.todo = b.todo_n = nullptr;
         b.retry_n = counters + 3;
-        b.retry = sc.get<unsigned int>(k <= 66 ? idx->cnt[0] : 1);
+        b.retry = sc.get<unsigned int>(k <= 92 ? idx->cnt[0] : 1);
         b.beyond_n = counters + 4;
         b.beyond = sc.get<unsigned int>(idx->cnt[0]);
         b.work = d_work;
         SF_TRY_SCRATCH(sc);
-        if (k <= 66) {
+        if (k <= 92) {
             if (k <= 34) SF_TRY((launch_sel<96, 13>(b, idx->cnt[0], sc, s)));
             else SF_TRY((launch_sel<144, 10>(b, idx->cnt[0], sc, s)));
             b.todo = b.retry;

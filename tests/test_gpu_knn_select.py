@@ -53,3 +53,9 @@ def test_knn_bit_exact(cloud, n, k):
     ref, _, _ = oracle.knn(xyz, k)
     assert np.array_equal(h.cpu().numpy().view(np.uint32), np.asarray(ref, dtype=np.float32).view(np.uint32))
     assert work["query_leaves"] == -(-n // 32)
+
+
+@pytest.mark.parametrize("cloud", sorted(CLOUDS))
+@pytest.mark.parametrize("n,k", [(94, 92), (95, 93), (2500, 79), (3001, 92), (3001, 93)])
+def test_knn_where_the_longest_lists_begin(cloud, n, k):
+    test_knn_bit_exact(cloud, n, k)
