@@ -1034,8 +1034,16 @@ struct KnnSel {
                 }
             }
         }
-        if (found && !(dk > 1.0e-34f && dk < 1.0e37f)) ok = false;
-        if (found && ok) {
+        // d2 = 0 in FP32: the k-th coincides with the query, or FP32 does not show how far it is
+        int zero = 0;
+        if (found && dk == 0.f)
+            for (int i = 0; i < nmem; ++i) {
+                const float4 p = __ldg(&tv.pos[point_of(S.list[i][lane])]);
+                zero += p.x == q.x && p.y == q.y && p.z == q.z;
+            }
+        const bool at_zero = found && dk == 0.f && zero >= need;
+        if (found && !at_zero && !(dk > 1.0e-34f && dk < 1.0e37f)) ok = false;
+        if (found && ok && !at_zero) {
             kth = d2_f64(q, __ldg(&tv.pos[at]));
             if (ties > 1) {  // rank them in FP64, from one value to the next (exact ties are one)
                 kth = -1.0;

@@ -109,3 +109,15 @@ def test_coinciding(each, k, apart):
     if apart == "near":
         p[:, 2] = 1e-24 * r.integers(0, 3, n)
     _check(p, k)
+
+
+@pytest.mark.parametrize("k", [1, 2, 8, 40, 100])
+@pytest.mark.parametrize("heavy", [3, 20, 700, 5000])
+def test_coinciding_among_close_neighbours(heavy, k):
+    """Points at one place among others a rounding of the coordinates away (all within one cell
+    of the index's order, so they do not follow one another in it): k-th distances of 0 and
+    of one rounding, some at the place, some beside it with too few of their own."""
+    r = np.random.default_rng(heavy + k)
+    ulp = float(np.spacing(F(0.5)))
+    around = 0.5 + ulp * r.integers(-3, 4, (600, 3))
+    _check(np.concatenate([np.full((heavy, 3), 0.5), around, r.random((1500, 3))])[r.permutation(heavy + 2100)], k)
