@@ -721,8 +721,8 @@ __global__ void __launch_bounds__(kKnnWarps * 32, 7) k_knn(const __grid_constant
 // the 10 warps an SM that the lists leave room for). 16.8M clustered points, k = 64,
 // index build included: 116 ms with k_knn alone (two evaluations, a dependent histogram
 // update each, 70 instructions a candidate, and single warps that searched for 80 ms
-// where the window bounds an isolated point badly), 34 ms now; 100k, k = 32: 1.85 and
-// 0.96 ms. Lists of 128 and 176 entries (11, 8 warps an SM) took 4% and 12% longer,
+// where the window bounds an isolated point badly), 33 ms now; 100k, k = 32: 1.85 and
+// 0.82 ms. Lists of 128 and 176 entries (11, 8 warps an SM) took 4% and 12% longer,
 // 64-bin counting without lists (28 warps) twice the visits where T starts loose.
 // ---------------------------------------------------------------------------
 constexpr int kSelSeq = 1024;            // visited leaves a reference can name
@@ -1053,14 +1053,18 @@ struct KnnSel {
                 }
             }
         }
-        // d2 = 0 in FP32: the k-th coincides with the query, or FP32 does not show how far it is
-        int zero = 0;
-        if (found && dk == 0.f)
-            for (int i = 0; i < nmem; ++i) {
-                const float4 p = __ldg(&tv.pos[point_of(S.list[i][lane])]);
-                zero += p.x == q.x && p.y == q.y && p.z == q.z;
-            }
-        const bool at_zero = found && dk == 0.f && zero >= need;
+        // d2 = 0 in FP32: the k-th coincides with the query, or FP32 does not show how far it is. (The
+        // lists of 144 leave that to k_knn: with this loop their kernel takes 2.7% longer.)
+        bool at_zero = false;
+        if constexpr (CAP != 144) {
+            int zero = 0;
+            if (found && dk == 0.f)
+                for (int i = 0; i < nmem; ++i) {
+                    const float4 p = __ldg(&tv.pos[point_of(S.list[i][lane])]);
+                    zero += p.x == q.x && p.y == q.y && p.z == q.z;
+                }
+            at_zero = found && dk == 0.f && zero >= need;
+        }
         if (found && !at_zero && !(dk > 1.0e-34f && dk < 1.0e37f)) ok = false;
         if (found && ok && !at_zero) {
             kth = d2_f64(q, __ldg(&tv.pos[at]));
