@@ -70,23 +70,32 @@ __device__ __forceinline__ float mix2(float ah, float al, float bh, float bl, co
     return r;
 }
 
-// The same in FP64, for nodes that the float pairs cannot settle.
-__device__ __noinline__ float resample_fp64(const float *__restrict__ f, int64_t row, int64_t slice, double ux,
-                                            double uy, double uz, float weight) {
-    const double vx = 1.0 - ux, vy = 1.0 - uy, vz = 1.0 - uz;
-    const double w[4] = {vx * vy, ux * vy, vx * uy, ux * uy};
+// float to double by its bits (the conversion instruction runs at the FP64 rate, a 64th of FP32's: 2 x 4096 x 1024 nodes in FP64 0.57 ms with it, 0.38 so).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u) return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    return m == 0u ? __hiloint2double((int)u, 0) : (double)f;
+}
+
+// The same in FP64, for nodes that the float pairs cannot settle (x, y, z: the weights of the
+// cell's lower and upper node).
+__device__ __noinline__ float resample_fp64(const float *__restrict__ f, int64_t row, int64_t slice, double2 x,
+                                            double2 y, double2 z, float weight) {
+    const double w[4] = {x.x * y.x, x.y * y.x, x.x * y.y, x.y * y.y};
     double val = 0.0;
 #pragma unroll
     for (int t = 0; t < 8; ++t)
-        val += w[t & 3] * (t >> 2 ? uz : vz) * (double)__ldg(f + (t & 1) + ((t >> 1) & 1) * row + (t >> 2) * slice);
-    return (float)((double)weight * val);
+        val += w[t & 3] * (t >> 2 ? z.y : z.x) * widen(__ldg(f + (t & 1) + ((t >> 1) & 1) * row + (t >> 2) * slice));
+    return (float)(widen(weight) * val);
 }
 
 // What bounds it: with every node's cell, weights and sum in FP64 (about 70 instructions
 // at 2 lanes a clock and SM) it ran at the FP64 rate: 108 us for 96^3 nodes. Per-axis
 // places (one FP64 evaluation per block and axis node) leave the sum, about 120 FP32
-// instructions in float pairs: 8.8 us (11 with cold caches), bounded by issue and the blocks' start-up (7.4 MB of
-// compulsory traffic would take 1.1 us). Settling the rounding costs about 0.7 us of that (calls in a row: 10.25 and 10.9 us). The pairs are good to 2^-41.8 of a sum of
+// instructions in float pairs: 8.8 us (11 with cold caches), bounded by issue and the blocks'
+// start-up (7.4 MB of compulsory traffic would take 1.1 us). Settling the rounding costs one to
+// two us of a call (in a row: 10.3 us without, 11.3 to 12.3 with), the time that the ten or so
+// open nodes of 96^3 take in FP64, each on its own. The pairs are good to 2^-41.8 of a sum of
 // non-negative terms (2^-45.3, 2^-43.6 and 2^-42.9 for the three steps, whose low parts grow
 // to 2^-20.7; 2^-44.7 for the weight; 2^-48 a pair of weights); kRsError covers that and the
 // 2^-49 of FP64, so where both ends of the interval round to one float, FP64 rounds to
@@ -94,17 +103,19 @@ __device__ __noinline__ float resample_fp64(const float *__restrict__ f, int64_t
 constexpr float kRsError = 0x1p-41f;
 // A block takes 256 columns of up to 8 nodes. A warp is 32 nodes wide in x, or narrower (8, in
 // grids narrower than that 2) where an eighth fewer warps cover the grid so (2 x 4096 x 1024
-// nodes of a signed field, all FP64: 14.5 ms with 32 always, 0.57 now; 33 x 300 x 300: 397
-// us and 260). Columns are shorter where the blocks would not fill the chip (33^3 nodes of a signed
+// nodes of a signed field, all FP64: 14.5 ms with 32 always, 0.38 now; 33 x 300 x 300: 397
+// us and 177). Columns are shorter where the blocks would not fill the chip (33^3 nodes of a signed
 // field: 41 us a call with 8, 26 now).
 constexpr int kRsThreads = 256, kRsZ = 8;
 constexpr int kRsBlocks = 2 * 152;
 
+template <bool TALL>
 __global__ void __launch_bounds__(kRsThreads)
-    k_resample(const float *__restrict__ src, Axes A, int xlog, int zlen, float weight, int accumulate, float *__restrict__ dst,
+    k_resample(const float *__restrict__ src, Axes A, int xlog, int z_nodes, float weight, int accumulate, float *__restrict__ dst,
                unsigned long long *outside) {
     __shared__ AxisPlace P[kRsThreads];  // of the block's nodes in x, y and z
-    __shared__ double U[kRsThreads];     // their FP64 places in the cell
+    __shared__ double2 U[kRsThreads];    // their weights in FP64
+    const int zlen = TALL ? kRsZ : z_nodes;  // (a constant saves 1 us of 12 at 96^3)
     const int tid = threadIdx.x, bx = 1 << xlog, by = kRsThreads >> xlog;
     const int g0[3] = {(int)blockIdx.x * bx, (int)blockIdx.y * by, (int)blockIdx.z * zlen};
     if (tid < bx + by + zlen) {
@@ -114,7 +125,7 @@ __global__ void __launch_bounds__(kRsThreads)
         bool in;
         const double u = axis_cell(A, k, i, p.c, in), v = 1.0 - u;
         if (!in) p.c = -1;
-        U[tid] = u;
+        U[tid] = make_double2(v, u);
         p.w0h = (float)v;
         p.w0l = (float)(v - (double)p.w0h);
         p.w1h = (float)u;
@@ -228,7 +239,7 @@ extern "C" sf_status sf_resample_grid(const float *d_src, const sf_box *src_box,
     const int bx = ceil_div(A.dn[0], 1 << xlog), by = ceil_div(A.dn[1], kRsThreads >> xlog);
     while (zlen > 1 && (int64_t)bx * by * ceil_div(A.dn[2], zlen) < kRsBlocks) zlen /= 2;
     const dim3 grid(bx, by, ceil_div(A.dn[2], zlen));
-    SF_TRY_CUDA(launch(k_resample, grid, dim3(kRsThreads), 0, s, d_src, A, xlog, zlen, weight, accumulate ? 1 : 0, d_dst, cnt));
+    SF_TRY_CUDA(launch(zlen == kRsZ ? k_resample<true> : k_resample<false>, grid, dim3(kRsThreads), 0, s, d_src, A, xlog, zlen, weight, accumulate ? 1 : 0, d_dst, cnt));
     if (h_outside) {
         unsigned long long h = 0;
         SF_TRY_CUDA(cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, s));
