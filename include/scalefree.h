@@ -171,7 +171,9 @@ int64_t sf_index_size(const sf_index *idx);
  * same rule. The kernels are queued on `stream` and the call returns without
  * waiting for them: a later call on another stream must be ordered after them
  * (an event, or a synchronisation) -- streams created non-blocking do not wait
- * for the legacy default stream.
+ * for the legacy default stream. Scratch of the kNN rule, not part of
+ * sf_query_workspace: 8 bytes per 32 points and the resident warps' lists
+ * (about 0.25 GB in all, less for small clouds).
  */
 sf_status sf_bandwidths(sf_index *idx, const sf_params *params, void *stream);
 

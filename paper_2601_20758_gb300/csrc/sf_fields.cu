@@ -70,7 +70,8 @@ __device__ __forceinline__ float mix2(float ah, float al, float bh, float bl, co
     return r;
 }
 
-// float to double by its bits (the conversion instruction runs at the FP64 rate, a 64th of FP32's: 2 x 4096 x 1024 nodes in FP64 0.57 ms with it, 0.38 so).
+// float to double by its bits (the conversion instruction runs at the FP64 rate, a 64th of FP32's:
+// 2 x 4096 x 1024 nodes in FP64 took 0.57 ms with it, 0.38 so).
 __device__ __forceinline__ double widen(float f) {
     const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
     if (m - 0x00800000u < 0x7f000000u) return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
